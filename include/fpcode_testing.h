@@ -109,6 +109,18 @@ int fpcode_test_tune_search(int ndim, const int *sizes, const int *start, const 
  * and *j receive its level and information set.  Returns 0, or -1 if the
  * key names no codeword of the schedule. */
 int fpcode_test_key_coefficients(const fpcode_prepared *prep, uint64_t key, int *g, int *j, int *coef);
+/* fpcode_prepare for the tensor-core kernel whatever the expected size of
+ * the search (opts->pair_leaves = 2).  FPCODE_EINVAL if that kernel does not
+ * take the code. */
+int fpcode_test_prepare_split(int p, int n, int k, const uint8_t *G, const fpcode_opts *opts, fpcode_prepared **out);
+/* The codewords a split pass (the tensor-core kernel's walk) visits, in its
+ * order, as packed keys of weight 0 in the code's leaf form: the pass's own
+ * tasks planned for `ctas` CTAs (tail_rows = 0), or the whole pass with
+ * tails of tail_rows rows in blocks of `block`, `unit` stems per lane and
+ * 1 << esplit slices.  Returns their number (entries past max not
+ * written), or -1 (no such pass, or the code is not searched this way). */
+int64_t fpcode_test_split_pass(fpcode_prepared *prep, int pass, int ctas, int tail_rows, int block, int unit, int esplit,
+                               uint64_t *keys, int64_t max);
 /* Microseconds from the start of the last search on `prep` to the end of
  * each of its passes (-1: not reached), for up to max passes.  Returns the
  * number of passes written, or -1. */

@@ -198,6 +198,11 @@ def _declare(lib):
         "fpcode_test_lane_ranges": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                    ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64),
                                                    ctypes.c_int]),
+        "fpcode_test_prepare_split": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, _U8P,
+                                                     ctypes.POINTER(fpcode_opts), ctypes.POINTER(_VP)]),
+        "fpcode_test_split_pass": (ctypes.c_int64, [_VP, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int,
+                                                    ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_uint64),
+                                                    ctypes.c_int64]),
         "fpcode_test_pair_table_device": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.POINTER(ctypes.c_uint32), ctypes.c_int]),
         "fpcode_prepared_pass_slice": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_uint64, ctypes.c_uint64, ctypes.c_int,
                                                       ctypes.POINTER(_VP)]),
@@ -830,6 +835,25 @@ def fpcode_test_pair_table_device(prep: Prepared, j: int) -> np.ndarray:
     if n < 0:
         raise FpcodeError(-n, "fpcode_test_pair_table_device")
     return out[:n].copy()
+
+
+def fpcode_test_prepare_split(p: int, n: int, k: int, G, opts: fpcode_opts) -> Prepared | None:
+    """fpcode_prepare for the tensor-core kernel whatever the search's size,
+    or None if that kernel does not take the code."""
+    G = _matrix(G)
+    h = _VP()
+    st = lib().fpcode_test_prepare_split(p, n, k, G.ctypes.data_as(_U8P), ctypes.byref(opts), ctypes.byref(h))
+    return None if _check(st, "fpcode_test_prepare_split", ok=(OK, EINVAL)) else Prepared(h.value, p, n, k)
+
+
+def fpcode_test_split_pass(prep: Prepared, pass_index: int, ctas: int = 152, tail_rows: int = 0, block: int = 96,
+                           unit: int = 1, esplit: int = 0, cap: int = 1 << 22) -> np.ndarray | None:
+    """Packed keys (weight 0) of the codewords a split pass visits, or None
+    if the code is not searched by the tensor-core kernel."""
+    keys = np.zeros(cap, dtype=np.uint64)
+    n = lib().fpcode_test_split_pass(prep.handle, int(pass_index), int(ctas), int(tail_rows), int(block), int(unit),
+                                     int(esplit), keys.ctypes.data_as(ctypes.POINTER(ctypes.c_uint64)), cap)
+    return None if n < 0 else keys[:min(n, cap)]
 
 
 def fpcode_test_key_coefficients(prep: Prepared, key: int):

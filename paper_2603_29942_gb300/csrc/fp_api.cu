@@ -112,14 +112,14 @@ const void *kernel_for(int variant) {
 }
 
 // CTAs per SM for a kernel with `smem` bytes of dynamic shared memory.
-int occupancy(const void *fn, int smem, int override_per_sm, int *per_sm) {
+int occupancy(const void *fn, int smem, int override_per_sm, int *per_sm, int threads) {
   cudaFuncAttributes fa{};
   FP_CUDA(cudaFuncGetAttributes(&fa, fn));
   // dynamic and static shared memory together past 48 KiB need the opt-in
   if ((size_t)smem + fa.sharedSizeBytes > 48 * 1024)
     FP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   int n = 0;
-  FP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, fpk::kThreads, (size_t)smem));
+  FP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, (size_t)smem));
   if (n < 1) {
     fph::set_error("kernel cannot be resident (shared memory or registers)");
     return FPCODE_EINVAL;
@@ -162,6 +162,14 @@ struct Layout {
   std::vector<size_t> pass_off, table_off;
 };
 
+// A code's plan segments: those of the tensor-core kernel or of pair leaves.
+size_t segs_bytes(const fph::Prepared &P) {
+  return P.split ? P.split_segs.size() * sizeof(fpk::SplitSeg) : P.segs.size() * sizeof(fpk::PairSeg);
+}
+const void *segs_data(const fph::Prepared &P) {
+  return P.split ? (const void *)P.split_segs.data() : (const void *)P.segs.data();
+}
+
 Layout make_layout(const std::vector<const fph::Prepared *> &codes) {
   Layout L;
   const size_t ns = codes.size();
@@ -173,7 +181,7 @@ Layout make_layout(const std::vector<const fph::Prepared *> &codes) {
   L.off_passes = o;
   for (auto *P : codes) {  // each code's passes, then its pair-leaf segments (read as passes + npasses)
     L.pass_off.push_back(o);
-    o = align256(o + P->passes.size() * sizeof(PassDesc) + P->segs.size() * sizeof(fpk::PairSeg));
+    o = align256(o + P->passes.size() * sizeof(PassDesc) + segs_bytes(*P));
   }
   L.off_tables = o;
   for (auto *P : codes) {
@@ -228,14 +236,17 @@ void fill_static(const Layout &L, const std::vector<const fph::Prepared *> &code
     sd.seed_u = P.seed_u;
     sd.pair_sigp = P.pair ? P.pair_sigp : 0;
     sd.pair_quick_max = P.pair_quick_max;
-    sd.nsegs = (int)P.segs.size();
+    sd.nsegs = (int)(P.split ? P.split_segs.size() : P.segs.size());
+    if (P.split) {
+      sd.split_k = P.split_k;
+      sd.split_nu = P.split_nu;
+      sd.split_cap = P.split_cap;
+    }
     sd.table = reinterpret_cast<const uint32_t *>(d + L.table_off[i]);
     sd.passes = reinterpret_cast<const PassDesc *>(d + L.pass_off[i]);
     std::memcpy(h + L.off_slots + i * sizeof(SlotDesc), &sd, sizeof(sd));
     std::memcpy(h + L.pass_off[i], P.passes.data(), P.passes.size() * sizeof(PassDesc));
-    if (!P.segs.empty())
-      std::memcpy(h + L.pass_off[i] + P.passes.size() * sizeof(PassDesc), P.segs.data(),
-                  P.segs.size() * sizeof(fpk::PairSeg));
+    if (segs_bytes(P)) std::memcpy(h + L.pass_off[i] + P.passes.size() * sizeof(PassDesc), segs_data(P), segs_bytes(P));
     std::memcpy(h + L.table_off[i], P.table.data(), P.table.size() * sizeof(uint32_t));
   }
 }
@@ -255,14 +266,15 @@ fph::DeviceOutcome outcome_of(const SlotState &s, const CtlDyn &dyn) {
   return o;
 }
 
-int launch(const void *fn, int ctas, int smem, cudaStream_t st, char *d, const Layout &L, const KParams &kp) {
+int launch(const void *fn, int ctas, int smem, cudaStream_t st, char *d, const Layout &L, const KParams &kp,
+           int threads = fpk::kThreads) {
   const SlotDesc *slots = reinterpret_cast<const SlotDesc *>(d + L.off_slots);
   SlotState *states = reinterpret_cast<SlotState *>(d + L.off_states);
   const CtlStatic *ctl = reinterpret_cast<const CtlStatic *>(d + L.off_ctl);
   CtlDyn *dyn = reinterpret_cast<CtlDyn *>(d + L.off_states + L.dyn_bytes - sizeof(CtlDyn));
   KParams kpv = kp;
   void *args[] = {(void *)&slots, (void *)&states, (void *)&ctl, (void *)&dyn, (void *)&kpv};
-  FP_CUDA(cudaLaunchKernel(fn, dim3(ctas), dim3(fpk::kThreads), args, (size_t)smem, st));
+  FP_CUDA(cudaLaunchKernel(fn, dim3(ctas), dim3(threads), args, (size_t)smem, st));
   return FPCODE_OK;
 }
 
@@ -274,6 +286,12 @@ int smem_for(const std::vector<const fph::Prepared *> &codes) {
   return (int)(((s + 15) & ~(size_t)15) + fpk::kBinomBytes);
 }
 
+// Kernel of a one-code launch, and its threads per CTA.
+const void *kernel_of(const fph::Prepared &P) {
+  return P.split ? fpk::kernel_split(P.p, P.W) : kernel_for(P.variant);
+}
+int threads_of(const fph::Prepared &P) { return P.split ? fpk::kSplitThreads : fpk::kThreads; }
+
 // with_state: the host image also holds the first state (zeroed
 // bookkeeping, the bound in the best key) and one copy takes both, so the
 // next search needs no reset of its own.
@@ -281,18 +299,21 @@ int smem_for(const std::vector<const fph::Prepared *> &codes) {
 // segments are part of the static image).
 int plan_one(fpcode_prepared *prep, const DevCtx &c) {
   fph::Prepared &P = prep->host;
-  const void *fn = kernel_for(P.variant);
+  const void *fn = kernel_of(P);
   if (!fn) {
     fph::set_error("no kernel for this (p, n - k)");
     return FPCODE_EINVAL;
   }
-  prep->smem = smem_for({&P});
+  prep->smem = P.split ? fph::split_smem_bytes(P) : smem_for({&P});
   int per_sm = 0;
-  int s = occupancy(fn, prep->smem, P.opts.ctas_per_sm, &per_sm);
+  int s = occupancy(fn, prep->smem, P.opts.ctas_per_sm, &per_sm, threads_of(P));
   if (s) return s;
   prep->ctas = c.sms * per_sm;
-  fph::plan_tasks(&P, prep->ctas, P.opts.prefixes_per_lane, P.opts.min_steps > 0 ? P.opts.min_steps : fph::kMinStepsSingle,
-                  true);
+  if (P.split)
+    fph::plan_split(&P, prep->ctas);
+  else
+    fph::plan_tasks(&P, prep->ctas, P.opts.prefixes_per_lane,
+                    P.opts.min_steps > 0 ? P.opts.min_steps : fph::kMinStepsSingle, true);
   if (prep->slice_hi > 0) {  // a slice of the one pass: its tasks under the same plan
     fpk::PassDesc &d = P.passes[0];
     const uint64_t hi = std::min<uint64_t>(prep->slice_hi, d.ntasks);
@@ -376,7 +397,7 @@ int enqueue_one(fpcode_prepared *prep, cudaStream_t st, const fpcode_opts &o) {
   }
   if (!P.passes.empty()) {
     FP_CUDA(cudaEventRecord((cudaEvent_t)prep->ev0, st));
-    int s = launch(kernel_for(P.variant), prep->ctas, prep->smem, st, prep->dev, L, kparams(o, 0));
+    int s = launch(kernel_of(P), prep->ctas, prep->smem, st, prep->dev, L, kparams(o, 0), threads_of(P));
     if (s) return s;
     FP_CUDA(cudaEventRecord((cudaEvent_t)prep->ev1, st));
   }
@@ -689,6 +710,7 @@ int fpcode_min_distance_batch(int num, const fpcode_desc *codes, void *stream, c
         if (!per_variant) oi.pair_leaves = 0;  // the batched kernels take one-row leaves
         if (codes[i].budget) oi.budget = codes[i].budget;
         status[i] = fph::prepare(codes[i].p, codes[i].n, codes[i].k, codes[i].G, oi, preps[i].get());
+        preps[i]->split = false;  // many codes share a launch: the leaf kernels
       }
     };
     std::vector<std::thread> pool;

@@ -29,7 +29,7 @@ int get_ctx(DevCtx **out);
 // Kernel of one (prime class, words) variant.
 const void *kernel_for(int variant);
 // CTAs per SM for `fn` with `smem` bytes of dynamic shared memory.
-int occupancy(const void *fn, int smem, int override_per_sm, int *per_sm);
+int occupancy(const void *fn, int smem, int override_per_sm, int *per_sm, int threads = fpk::kThreads);
 // Per-launch limits from the options.
 fpk::KParams kparams(const fpcode_opts &o, int serve);
 

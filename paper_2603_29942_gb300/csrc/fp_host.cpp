@@ -7,6 +7,7 @@
 #include <cmath>
 #include <chrono>
 #include <cstring>
+#include <new>
 #include <unordered_map>
 #include <string>
 #include <vector>
@@ -240,11 +241,20 @@ double expected_work(int p, int n, int k) {
   if (memo.size() < 4096) memo.emplace(key, w);
   return w;
 }
+// Tensor-core kernel (pair_leaves 2): from this much expected work on, and
+// with at least this many redundant symbols (its class comparison needs
+// some).  Measured per call, leaf kernels against it: F_7 [40,20] (4.2e7
+// codewords) 80 against 112 us, F_3 [80,40] (2.7e8) 177 against 161, F_5
+// [51,24] (3.0e8) 429 against 169, F_7 [52,19] (2.9e10) 17 400 against 2 890.
+constexpr double kSplitWork = 1e8;
+constexpr int kSplitMinRed = 4;
+// Dynamic shared memory of one of its CTAs: 227 KiB less the kernel's own.
+constexpr int kSplitSmemMax = 218000;
 constexpr double kPairWork = 1e8;  // pair_leaves 2: pair leaves from this much expected work on
 
 }  // namespace
 
-int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prepared *P) {
+int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prepared *P, bool any_size) {
   auto t0 = std::chrono::steady_clock::now();
   if (!is_odd_prime(p)) {
     set_error("p must be an odd prime below 256");
@@ -478,6 +488,26 @@ int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prep
     if (P->passes.size() > round_start && !truncated) P->passes.back().round_end = 1;
   }
   P->complete = truncated ? 0 : 1;
+  // The tensor-core kernel takes the code when the leaf form is left to the
+  // library, its class values fit a row, a useful number of tails fits
+  // beside them, and the search is large: expected to be, and not cut short
+  // by its budget.
+  P->split = false;
+  P->split_k = P->split_nu = P->split_cap = 0;
+  if (opts.pair_leaves == 2 && (p == 3 || p == 5 || p == 7) && k >= 3 && n - k >= kSplitMinRed &&
+      (any_size || std::min((double)total, expected_work(p, n, k)) >= kSplitWork)) {
+    const int K = fpk::split_k(p, n - k, &P->split_nu);
+    if (K > 0) {
+      const int room = kSplitSmemMax - fpk::split_off_tails(k, p, P->rwpad) - 128;
+      const int cap = room / (K + 4) / fpk::kSplitN * fpk::kSplitN;
+      const uint64_t most = fpk::tails_above(binom(), k, 3, p - 1, -1);
+      const int need = (int)std::min<uint64_t>((std::max<uint64_t>(most, fpk::tails_above(binom(), k, 2, p - 1, -1)) +
+                                                fpk::kSplitN - 1) / fpk::kSplitN * fpk::kSplitN, 1u << 20);
+      P->split_cap = std::min(cap, need);
+      P->split_k = K;
+      P->split = cap >= 4 * fpk::kSplitN;
+    }
+  }
   // The g = 1 passes are the rows of the Gamma_j themselves: their least
   // weight is known now.  A search starts with it as its bound (the claims
   // cap U with it; no key stands behind it), so the tasks that start at once
@@ -706,6 +736,197 @@ void plan_tasks(Prepared *P, int ctas, int fixed_pl, int min_steps, bool spread_
     d.phases = H;
   }
   // one task sequence over all passes
+  uint64_t base = 0;
+  for (auto &d : P->passes) {
+    d.task_base = (uint32_t)base;
+    base += d.ntasks;
+  }
+}
+
+int split_smem_bytes(const Prepared &P) {
+  // at least half of an SM's shared memory, so that a second such CTA, which
+  // would wait for the first one's tensor memory, never becomes resident
+  return std::max(fpk::split_smem(P.k, P.p, P.rwpad, P.split_cap, P.split_k), 120 * 1024);
+}
+
+namespace {
+
+// Issue slots of the tensor-core kernel (per warp scheduler, one warpgroup
+// at work on it): a stem's step and class values, the start of a lane's run
+// of stems, one tile of results, and the build of a block of n tails.
+constexpr double kStemSlots = 150, kRunSlots = 400, kTileSlots = 85;
+inline double build_slots(double n) { return 1000 + 0.9 * n; }
+constexpr double kTaskSlots = 5000;        // least work of a task, so that claims stay a small part
+constexpr uint64_t kDirectCombos = 1 << 19;  // stem-tail pairs of a pass up to which every weight is computed exactly
+
+// Stems of pass level g with tails of t rows whose largest row is below z.
+uint64_t stems_below(const Prepared &P, int z, int l, uint64_t ncl) { return l > 0 ? binom().c[z][l] * ncl : 1; }
+
+struct SplitCost {
+  double slots = 0;  // of all warpgroups
+  int blocks = 0;
+};
+// Work of a pass with tails of t rows in blocks of nb.
+SplitCost split_cost(const Prepared &P, int g, int t, uint32_t nb, uint64_t ncl) {
+  const int k = P.k, b = P.p - 1, l = g - t;
+  const uint32_t etot = fpk::tails_above(binom(), k, t, b, -1);
+  SplitCost c;
+  for (uint32_t first = 0; first < etot; first += nb) {
+    ++c.blocks;
+    const uint32_t n = std::min(nb, etot - first);
+    const int m = fpk::comb_floor(binom(), t - 1, k - 1, t, fpk::tail_coefs(t, b), first);
+    const int zhi = k - 1 - m;
+    if (l == 0) {
+      c.slots += kRunSlots + kTileSlots * ((n + fpk::kSplitN - 1) / fpk::kSplitN);
+      continue;
+    }
+    if (t == 3) {  // a few values of z to a block: every stem meets most of it
+      c.slots += (double)stems_below(P, zhi, l, ncl) / 128 * (kStemSlots + kTileSlots * (double)((n + fpk::kSplitN - 1) / fpk::kSplitN));
+      continue;
+    }
+    for (int q = l - 1; q < zhi; ++q) {
+      const uint32_t e = std::min(n, fpk::tails_above(binom(), k, t, b, q) - first);
+      c.slots += (double)(binom().c[q][l - 1] * ncl) / 128 * (kStemSlots + kTileSlots * (double)((e + fpk::kSplitN - 1) / fpk::kSplitN));
+    }
+  }
+  return c;
+}
+
+}  // namespace
+
+// Every pass with g >= 2 gets its tail length, block size and runs of
+// tasks.  Tails of three rows serve a stem more entries (their blocks are
+// full but for the stem's step), tails of two need fewer tables; the
+// cheaper of the two by the slots above.
+void plan_split(Prepared *P, int ctas) {
+  const double C = std::max(1, ctas);
+  const int k = P->k, b = P->p - 1;
+  P->split_segs.clear();
+  for (auto &d : P->passes) {
+    d.phases = 0;
+    d.plan_ctas = (uint32_t)ctas;
+    d.unit = 1;
+    d.pl = 0;
+    d.seg_off = (uint32_t)P->split_segs.size();
+    d.nseg = 0;
+    d.direct = 0;
+    d.esplit = 0;
+    d.tail_rows = 0;
+    d.block = 0;
+    d.ncl = 1;
+    if (d.g == 1) {
+      d.ntasks = 1;
+      continue;
+    }
+    const int g = d.g;
+    auto ncl_of = [&](int l) {
+      uint64_t v = l > 0 ? (uint64_t)(b / 2) : 1;
+      for (int i = 1; i < l; ++i) v *= (uint64_t)b;
+      return v;
+    };
+    int t = 2;
+    uint32_t nb = 0;
+    double total = 0;
+    const uint64_t combos = g == 2 ? d.size : d.size / 2;
+    if (combos <= kDirectCombos) {
+      d.direct = 1;
+      nb = fpk::tails_above(binom(), k, 2, b, -1);
+    } else {
+      double best = 0;
+      for (int tt = 2; tt <= 3; ++tt) {
+        if (tt == 3 && g < 4) break;
+        const uint32_t etot = fpk::tails_above(binom(), k, tt, b, -1);
+        for (int half = 0; half < (tt == 3 ? 2 : 1); ++half) {
+          const uint32_t cap = std::max<uint32_t>(fpk::kSplitN, (uint32_t)(P->split_cap >> half) / fpk::kSplitN * fpk::kSplitN);
+          const uint32_t nblk = (etot + cap - 1) / cap;
+          if (nblk > 255) continue;  // the run's field
+          const uint32_t size = ((etot + nblk - 1) / nblk + fpk::kSplitN - 1) / fpk::kSplitN * fpk::kSplitN;
+          const SplitCost c = split_cost(*P, g, tt, size, ncl_of(g - tt));
+          const double tasks = std::max<double>(c.blocks, std::min(C, c.slots / kTaskSlots));
+          const double cost = c.slots / C + build_slots(size) * std::max(1.0, tasks / C);
+          if (nb == 0 || cost < best) {
+            best = cost;
+            t = tt;
+            nb = size;
+            total = c.slots;
+          }
+        }
+      }
+    }
+    const int l = g - t;
+    d.tail_rows = (uint8_t)t;
+    d.block = nb;
+    d.ncl = ncl_of(l);
+    const uint32_t etot = fpk::tails_above(binom(), k, t, b, -1);
+    uint32_t tasks = 0;
+    auto add = [&](uint32_t item0, uint32_t item1, uint64_t per, uint32_t block, int zhi) {
+      if (item0 >= item1) return;
+      fpk::SplitSeg s{};
+      per = std::min<uint64_t>(std::max<uint64_t>(per, 1), 65535);
+      tasks += (uint32_t)((item1 - item0 + per - 1) / per);
+      s.task_end = tasks;
+      s.item0 = item0;
+      s.item1 = item1;
+      s.per = (uint16_t)per;
+      s.block = (uint8_t)block;
+      s.zhi = (uint8_t)zhi;
+      P->split_segs.push_back(s);
+    };
+    if (d.direct) {
+      d.esplit = g == 2 ? 2 : 0;
+      const uint32_t items = (uint32_t)(stems_below(*P, k - 2, l, d.ncl) << d.esplit);
+      add(0, items, std::max<uint64_t>(4, (uint64_t)((items + C - 1) / C)), 0, k - 2);
+    } else {
+      // stems per lane: long runs share the start of a lane, as long as the
+      // grid's warpgroups get eight items each
+      uint64_t stems = 0;
+      for (uint32_t first = 0, blk = 0; first < etot; first += nb, ++blk)
+        stems += stems_below(*P, k - 1 - fpk::comb_floor(binom(), t - 1, k - 1, t, fpk::tail_coefs(t, b), first), l, d.ncl);
+      uint32_t T = 1;
+      while (T < 32 && stems / (128 * 2 * T) >= (uint64_t)(8 * 4 * C)) T *= 2;
+      while (stems / (128ull * T) >= (1ull << 26)) T *= 2;  // items fit 32 bits with their slices
+      const uint32_t tiles_max = (std::min(nb, etot) + fpk::kSplitN - 1) / fpk::kSplitN;
+      int es = 0;
+      while (es < 4 && (stems / 128 << es) < (uint64_t)(4 * C) && (tiles_max >> es) >= 4) ++es;
+      d.unit = T;
+      d.esplit = (uint8_t)es;
+      double rem = total;
+      for (uint32_t first = 0, blk = 0; first < etot; first += nb, ++blk) {
+        const uint32_t n = std::min(nb, etot - first);
+        const int zhi = k - 1 - fpk::comb_floor(binom(), t - 1, k - 1, t, fpk::tail_coefs(t, b), first);
+        const uint64_t ns = stems_below(*P, zhi, l, d.ncl);
+        const uint32_t items = (uint32_t)(((ns + 128ull * T - 1) / (128ull * T)) << es);
+        // runs of items whose first stem meets the same number of tiles
+        uint32_t at = 0;
+        int q = std::max(l - 1, 0);
+        while (at < items) {
+          const uint32_t e = l > 0 ? std::min(n, fpk::tails_above(binom(), k, t, b, q) - first) : n;
+          const uint32_t tiles = (e + fpk::kSplitN - 1) / fpk::kSplitN;
+          int q1 = q + 1;
+          if (t == 3) q1 = zhi;
+          while (l > 0 && q1 < zhi &&
+                 (std::min(n, fpk::tails_above(binom(), k, t, b, q1) - first) + fpk::kSplitN - 1) / fpk::kSplitN == tiles)
+            ++q1;
+          uint32_t end = items;
+          if (l > 0 && q1 < zhi) end = std::min<uint32_t>(items, (uint32_t)((binom().c[q1][l] * d.ncl / (128ull * T)) << es));
+          if (end > at) {
+            const double per_item = kRunSlots + T * (kStemSlots + kTileSlots * std::max(1.0, (double)tiles / (1 << es)));
+            const double target = std::max(kTaskSlots, rem / (2 * C));
+            uint64_t per = (uint64_t)(target / per_item + 0.5);
+            if (per > 4) per = per / 4 * 4;  // the four warpgroups of a CTA share a task's items
+            if (per < 4) per = 4;
+            add(at, end, per, blk, zhi);
+            rem -= per_item * (end - at);
+            if (rem < 0) rem = 0;
+            at = end;
+          }
+          q = q1;
+        }
+      }
+    }
+    d.nseg = (uint32_t)P->split_segs.size() - d.seg_off;
+    d.ntasks = tasks;
+  }
   uint64_t base = 0;
   for (auto &d : P->passes) {
     d.task_base = (uint32_t)base;
@@ -1024,6 +1245,110 @@ int fpcode_test_key_coefficients(const fpcode_prepared *prep, uint64_t key, int 
   if (!fph::key_coefficients(prep->host, key, g, j, c)) return -1;
   for (int t = 0; t < prep->host.k; ++t) coef[t] = c[t];
   return 0;
+}
+
+extern "C++" {
+namespace {
+// The codewords of items [lo, hi) of one tail block, as the kernel walks
+// them (lanes in order, steps, tiles of the item's slice), as packed keys
+// of weight 0.
+template <int DB, class F>
+void split_walk(const fph::Prepared &P, const fpk::PassDesc &d, int pass, uint64_t lo, uint64_t hi, uint32_t block,
+                int zhi, F emit) {
+  const fpenum::Binom &B = fph::binom();
+  const int k = P.k, b = P.p - 1, g = d.g, t = d.tail_rows, l = g - t;
+  const uint32_t etot = fpk::tails_above(B, k, t, b, -1), first = block * d.block;
+  const uint32_t nb = std::min(d.block, etot - first), slices = 1u << d.esplit;
+  const uint64_t ns = l > 0 ? B(zhi, l) * d.ncl : 1;
+  const uint32_t T = d.direct ? 1 : d.unit, lanes = d.direct ? 1 : fpk::kSplitGroup;
+  const uint32_t tile = d.direct ? fpk::kSplitGroup : fpk::kSplitN;
+  for (uint64_t item = lo; item < hi; ++item) {
+    const uint64_t J0 = (item >> d.esplit) * lanes * T;
+    const uint32_t slice = (uint32_t)item & (slices - 1);
+    if (J0 >= ns) continue;
+    const int q0 = l > 0 ? fpk::comb_floor(B, l - 1, k - t - 1, l, d.ncl, J0) : -1;
+    const uint32_t tiles = (std::min(nb, fpk::tails_above(B, k, t, b, q0) - first) + tile - 1) / tile;
+    for (uint32_t lane = 0; lane < lanes; ++lane) {
+      const uint64_t J = J0 + (uint64_t)lane * T;
+      const uint32_t nst = J < ns ? (uint32_t)std::min<uint64_t>(T, ns - J) : 0;
+      fpenum::Prefix pf{-1, 0, 0, 0};
+      uint64_t ci = 0, nq = 1;
+      if (nst && l > 0) {
+        pf = fpk::stem_unrank<DB>(B, J, k, t, l, b, d.ncl, &ci);
+        nq = B(pf.m, l - 1);
+      }
+      for (uint32_t i = 0; i < nst; ++i) {
+        for (uint32_t c = slice; c < tiles; c += slices)
+          for (uint32_t e = c * tile; e < std::min((c + 1) * tile, nb); ++e) {
+            const fpk::Tail a = fpk::tail_unpack(fpk::tail_pack(fpk::tail_unrank(B, first + e, k, t, b)));
+            if (a.z <= pf.m) continue;
+            for (int sign = 0; sign < (l > 0 ? 2 : 1); ++sign)
+              emit(fpk::split_key<DB>(B, P.pair, k, P.p, g, (uint32_t)pass, 0, pf, l, a, sign));
+          }
+        int dir = 1;
+        if (l > 0 && i + 1 < nst) fpk::stem_advance<DB>(B, pf, ci, nq, d.ncl, b, l, &dir);
+      }
+    }
+  }
+}
+}  // namespace
+}  // extern "C++"
+
+int fpcode_test_prepare_split(int p, int n, int k, const uint8_t *G, const fpcode_opts *opts, fpcode_prepared **out) {
+  if (!out || !opts) return FPCODE_EINVAL;
+  *out = nullptr;
+  fpcode_prepared *prep = new (std::nothrow) fpcode_prepared();
+  if (!prep) return FPCODE_ENOMEM;
+  const int s = fph::prepare(p, n, k, G, *opts, &prep->host, true);
+  if (s || !prep->host.split) {
+    delete prep;
+    return s ? s : FPCODE_EINVAL;
+  }
+  *out = prep;
+  return FPCODE_OK;
+}
+
+int64_t fpcode_test_split_pass(fpcode_prepared *prep, int pass, int ctas, int tail_rows, int block, int unit, int esplit,
+                               uint64_t *keys, int64_t max) {
+  if (!prep || !prep->host.split || pass < 0 || pass >= (int)prep->host.passes.size() || !keys) return -1;
+  fph::Prepared &P = prep->host;
+  fph::plan_split(&P, ctas);
+  fpk::PassDesc d = P.passes[pass];
+  if (d.g < 2) return -1;
+  const int k = P.k, b = P.p - 1;
+  int64_t n = 0;
+  auto emit = [&](uint64_t key) {
+    if (n < max) keys[n] = key;
+    ++n;
+  };
+  auto walk = [&](uint64_t lo, uint64_t hi, uint32_t blk, int zhi) {
+    if (fph::digit_bits_of(P.p) == 1) split_walk<1>(P, d, pass, lo, hi, blk, zhi, emit);
+    else split_walk<4>(P, d, pass, lo, hi, blk, zhi, emit);
+  };
+  if (tail_rows == 0) {  // the plan's own tasks
+    for (uint64_t t = 0; t < d.ntasks; ++t) {
+      uint64_t lo = 0, hi = 0;
+      const fpk::SplitSeg s = fpk::split_task(&P.split_segs[d.seg_off], (int)d.nseg, t, &lo, &hi);
+      walk(lo, hi, s.block, s.zhi);
+    }
+    return n;
+  }
+  const int l = d.g - tail_rows;
+  if (tail_rows < 2 || tail_rows > 3 || l < 0 || block < 1 || unit < 1 || esplit < 0) return -1;
+  d.direct = 0;
+  d.tail_rows = (uint8_t)tail_rows;
+  d.block = (uint32_t)block;
+  d.unit = (uint32_t)unit;
+  d.esplit = (uint8_t)esplit;
+  d.ncl = l > 0 ? (uint64_t)(b / 2) : 1;
+  for (int i = 1; i < l; ++i) d.ncl *= (uint64_t)b;
+  const uint32_t etot = fpk::tails_above(fph::binom(), k, tail_rows, b, -1);
+  for (uint32_t first = 0, blk = 0; first < etot; first += (uint32_t)block, ++blk) {
+    const int zhi = fpk::tail_unrank(fph::binom(), first, k, tail_rows, b).z;
+    const uint64_t ns = l > 0 ? fph::binom()(zhi, l) * d.ncl : 1;
+    walk(0, ((ns + 128ull * unit - 1) / (128ull * unit)) << esplit, blk, zhi);
+  }
+  return n;
 }
 
 int fpcode_prepared_shape(const fpcode_prepared *prep, int *m, int *kj, int *npasses, int *complete) {

@@ -8,6 +8,7 @@
 
 #include "../../include/fpcode.h"
 #include "fp_enum.cuh"
+#include "fp_split.cuh"
 #include "fp_types.h"
 
 namespace fph {
@@ -44,6 +45,12 @@ struct Prepared {
   bool pair = false;
   int pair_sigp = 0;             // words per pair entry (a power of two)
   std::vector<fpk::PairSeg> segs;  // all passes' segments (PassDesc.seg_off, nseg)
+  // Split passes (fp_split.cuh): the code is searched by the tensor-core
+  // kernel.  Keys, schedule and counts are those of the leaf form above.
+  bool split = false;
+  int split_k = 0, split_nu = 0;  // class values per row, positions compared
+  int split_cap = 0;             // tails a CTA holds at a time
+  std::vector<fpk::SplitSeg> split_segs;  // all passes' runs of tasks
   int complete = 0;              // schedule reaches the last level
   uint64_t code_hash = 0;        // hash of (p, n, k, per_round_check, defer, pair) and G: schedule and key layout
   int seed_u = 0;                // least weight of the g = 1 passes (rows of the Gamma_j), 0: none;
@@ -76,7 +83,8 @@ int task_share_of(const fpcode_opts &o, bool last);
 
 // Elimination, information sets, multiples, schedule.  Returns an fpcode
 // status; the error text is set on failure.
-int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prepared *out);
+// any_size: the tensor-core kernel also for a search too small for it (tests).
+int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prepared *out, bool any_size = false);
 
 // Tasks and prefixes per lane of every pass for a grid of `ctas` CTAs.
 // fixed_pl > 0: tasks of fixed_pl prefixes per lane everywhere.  Else a pass
@@ -89,6 +97,11 @@ int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prep
 // search run with a loose threshold, many exact leaves each, and sit on the
 // path to the first termination tests).
 void plan_tasks(Prepared *P, int ctas, int fixed_pl, int min_steps, bool spread_tiny);
+
+// The same for the tensor-core kernel (P->split), into P->split_segs.
+void plan_split(Prepared *P, int ctas);
+// Dynamic shared memory of one of its CTAs.
+int split_smem_bytes(const Prepared &P);
 
 // Pair-leaf table limit per information set: with the binomial columns it
 // keeps four 256-thread CTAs resident per SM.

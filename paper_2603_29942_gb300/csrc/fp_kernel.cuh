@@ -25,8 +25,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "fp_bitslice.cuh"
 #include "fp_enum.cuh"
+#include "fp_split.cuh"
 #include "fp_types.h"
 
 namespace fpk {
@@ -918,15 +921,20 @@ struct Claim {  // the task taken (its code's and pass's descriptors: the ClaimC
   int slot, pass, U, skip;
   unsigned int ndone;       // tasks of the pass this claim completes (skipped runs: more than one)
   int lsplit;               // pair-leaf passes: lanes per stem (log2, low 4 bits) | stems per group << 4
+  unsigned int block;       // split passes: block of tails (ulo, uhi: its items)
+  int zhi;                  // split passes: z of the block's first tail
 };
 
 // Shared-memory copy of pair-leaf segments: for a one-code launch, the
 // whole list of the code (staged by the CTA at its start, pass = -2), else
 // those of the pass thread 0 claims from (at most (p-1)/2 (k-2) <= 186).
 constexpr int kSegPass = 192;
-template <int N>
+constexpr int kSplitSegCache = 320;  // the split kernel's copies of segments and pass descriptors
+constexpr int kSplitPassCache = 24;
+template <int N, class S = PairSeg>
 struct SegCache {
-  PairSeg seg[N];
+  using Seg = S;
+  Seg seg[N];
   int slot, pass;               // whose (-1: none; pass -2: the whole list)
   unsigned long long gen;
 };
@@ -1032,30 +1040,38 @@ __device__ __forceinline__ void take(SlotState *st, const KParams &kp, bool serv
   o->task = t - cc.pd.task_base + cc.pd.task_off;
   o->lsplit = 0;
   if (cc.pd.g > 1 && cc.pd.nseg > 0) {
-    // pair-leaf pass: its segments from the CTA's copy of the whole list,
-    // else copied for this pass (eight loads in flight at a time)
-    const PairSeg *segs = sc.seg;
+    // pair-leaf or split pass: its segments from the CTA's copy of the whole
+    // list, else copied for this pass (eight loads in flight at a time)
+    using Seg = typename SC::Seg;
+    using V = typename std::conditional<sizeof(Seg) == 16, uint4, uint2>::type;
+    const Seg *segs = sc.seg;
     if (sc.slot == s && sc.gen == cc.gen && sc.pass == -2) {
       segs += cc.pd.seg_off;
     } else if (sc.slot != s || sc.gen != cc.gen || sc.pass != cc.P) {
-      const uint2 *src = reinterpret_cast<const uint2 *>(cc.sd.passes + cc.sd.npasses) + cc.pd.seg_off;
+      const V *src = reinterpret_cast<const V *>(cc.sd.passes + cc.sd.npasses) + cc.pd.seg_off;
       const int n = min((int)cc.pd.nseg, kSegPass);
       for (int i0 = 0; i0 < n; i0 += 8) {
-        uint2 v[8];
+        V v[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
           if (i0 + u < n) v[u] = __ldcg(src + i0 + u);
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          if (i0 + u < n) reinterpret_cast<uint2 *>(sc.seg)[i0 + u] = v[u];
+          if (i0 + u < n) reinterpret_cast<V *>(sc.seg)[i0 + u] = v[u];
       }
       sc.slot = s;
       sc.gen = cc.gen;
       sc.pass = cc.P;
     }
-    int ls = 0, spg = 1;
-    pair_task(cc.pd, segs, cc.sd.k, B, o->task, &o->ulo, &o->uhi, &ls, &spg);
-    o->lsplit = ls | (spg << 4);
+    if constexpr (std::is_same<Seg, SplitSeg>::value) {
+      const SplitSeg g = split_task(segs, (int)cc.pd.nseg, o->task, &o->ulo, &o->uhi);
+      o->block = g.block;
+      o->zhi = g.zhi;
+    } else {
+      int ls = 0, spg = 1;
+      pair_task(cc.pd, segs, cc.sd.k, B, o->task, &o->ulo, &o->uhi, &ls, &spg);
+      o->lsplit = ls | (spg << 4);
+    }
   } else if (cc.pd.g > 1) {
     task_range(cc.pd, o->task, &o->ulo, &o->uhi);
   } else {
@@ -1385,6 +1401,31 @@ __device__ __forceinline__ bool finish_task(const CtlStatic &cs, const KParams &
 }
 
 
+// One-code launch with an outcome copy: the last CTA to leave copies the
+// final state (the outcome and the count of every CTA's codewords) to
+// host-mapped memory and zeroes the dynamic state, so the next search of
+// the code needs no reset and its result no copy of its own.  Called by
+// every thread of every CTA, last.
+__device__ __forceinline__ void leave_launch(SlotState *states, const CtlStatic &cs, CtlDyn *cdyn) {
+  if (!cs.outcome) return;
+  const int tid = threadIdx.x, threads = blockDim.x;
+  __shared__ int s_last;
+  if (tid == 0) {
+    fence_acq_rel();  // release: this CTA's writes before its count
+    s_last = atomicAdd(&cdyn->exited, 1u) == gridDim.x - 1 ? 1 : 0;
+    if (s_last) fence_acq_rel();  // acquire: every CTA's writes
+  }
+  __syncthreads();
+  if (s_last) {
+    const uint4 *src = reinterpret_cast<const uint4 *>(states);
+    uint4 *dst = reinterpret_cast<uint4 *>(cs.outcome);
+    for (int i = tid; i < (int)(cs.dyn_bytes / 16); i += threads) dst[i] = __ldcg(src + i);
+    __syncthreads();
+    uint4 *z = reinterpret_cast<uint4 *>(states);
+    for (int i = tid; i < (int)(cs.clean_bytes / 16); i += threads) z[i] = make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+
 #ifndef FPK_MIN_BLOCKS
 #define FPK_MIN_BLOCKS 4  // CTAs per SM the register allocation is capped for
 #endif
@@ -1554,27 +1595,7 @@ __global__ void __launch_bounds__(kThreads, FPK_MIN_BLOCKS) bz_kernel(const Slot
       }
     }
   }
-  if (cs.outcome) {
-    // One-code launch: the last CTA to leave copies the final state (the
-    // outcome and the count of every CTA's codewords) to host-mapped memory
-    // and zeroes the dynamic state, so the next search of the code needs no
-    // reset and its result no copy of its own.
-    __shared__ int s_last;
-    if (tid == 0) {
-      fence_acq_rel();  // release: this CTA's writes before its count
-      s_last = atomicAdd(&cdyn->exited, 1u) == gridDim.x - 1 ? 1 : 0;
-      if (s_last) fence_acq_rel();  // acquire: every CTA's writes
-    }
-    __syncthreads();
-    if (s_last) {
-      const uint4 *src = reinterpret_cast<const uint4 *>(states);
-      uint4 *dst = reinterpret_cast<uint4 *>(cs.outcome);
-      for (int i = tid; i < (int)(cs.dyn_bytes / 16); i += kThreads) dst[i] = __ldcg(src + i);
-      __syncthreads();
-      uint4 *z = reinterpret_cast<uint4 *>(states);
-      for (int i = tid; i < (int)(cs.clean_bytes / 16); i += kThreads) z[i] = make_uint4(0u, 0u, 0u, 0u);
-    }
-  }
+  leave_launch(states, cs, cdyn);
 }
 
 }  // namespace fpk

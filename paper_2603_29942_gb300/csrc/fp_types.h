@@ -58,6 +58,14 @@ struct PassDesc {
   uint32_t seg_off;        // pair-leaf passes: first segment of the pass in the code's segment list
   uint32_t nseg;           // pair-leaf passes: its segments (0: a one-row-leaf pass)
   uint32_t task_off;       // a slice of the pass (fpcode_prepared_pass_slice): its first task in the pass's plan
+  // Split passes (fp_split.cuh; then seg_off and nseg count SplitSegs, and
+  // `unit` is the stems per lane and item).
+  uint64_t ncl;            // coefficient vectors per stem row subset
+  uint32_t block;          // tails per block
+  uint8_t tail_rows;       // rows of a tail (2 or 3)
+  uint8_t direct;          // 1: few codewords, every weight exact
+  uint8_t esplit;          // log2 of the slices of a block's tails that are items of their own
+  uint8_t pad0;
 };
 
 // Words per row of the pair-signature table (Mersenne p = 3, 7): for each
@@ -123,7 +131,7 @@ FPK_HD void task_range(const PassDesc &d, uint64_t t, uint64_t *lo, uint64_t *hi
   *lo = row0 * kThreads;
   *hi = (row0 + nrow) * kThreads < N ? (row0 + nrow) * kThreads : N;
 }
-static_assert(sizeof(PassDesc) == 80, "PassDesc layout");
+static_assert(sizeof(PassDesc) == 96, "PassDesc layout");
 
 // ---------------------------------------------------------------------------
 // Pair leaves (p = 3, 7).  A codeword of pass g >= 3 with rows T splits into
@@ -232,8 +240,11 @@ struct SlotDesc {
   const PassDesc *passes;        // npasses entries, device
   uint64_t seq;                  // serving: ticket of the code in this slot
   unsigned long long *pass_times;  // optional: %globaltimer at each pass end (device)
+  int32_t split_k, split_nu;     // split passes: class values per row (0: none), positions compared
+  int32_t split_cap;             // split passes: tails a CTA holds at a time
+  int32_t pad0;
 };
-static_assert(sizeof(SlotDesc) == 96, "SlotDesc layout");
+static_assert(sizeof(SlotDesc) == 112, "SlotDesc layout");
 
 // Dynamic state of one code, device memory (all zero = fresh).  Three
 // 128-byte lines keep apart what is written at different rates: the task
