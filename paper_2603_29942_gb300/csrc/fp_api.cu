@@ -290,7 +290,7 @@ int smem_for(const std::vector<const fph::Prepared *> &codes) {
 const void *kernel_of(const fph::Prepared &P) {
   return P.split ? fpk::kernel_split(P.p, P.W) : kernel_for(P.variant);
 }
-int threads_of(const fph::Prepared &P) { return P.split ? fpk::kSplitThreads : fpk::kThreads; }
+int threads_of(const fph::Prepared &P) { return P.split ? fpk::kSplitThreads + 32 : fpk::kThreads; }
 
 // with_state: the host image also holds the first state (zeroed
 // bookkeeping, the bound in the best key) and one copy takes both, so the

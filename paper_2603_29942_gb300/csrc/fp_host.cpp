@@ -498,14 +498,14 @@ int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prep
       (any_size || std::min((double)total, expected_work(p, n, k)) >= kSplitWork)) {
     const int K = fpk::split_k(p, n - k, &P->split_nu);
     if (K > 0) {
-      const int room = kSplitSmemMax - fpk::split_off_tails(k, p, P->rwpad) - 128;
-      const int cap = room / (K + 4) / fpk::kSplitN * fpk::kSplitN;
+      const int room = kSplitSmemMax - fpk::split_off_tails(k, p, P->rwpad) - 256;
+      const int cap = std::max(room, 0) / (K + 4) / fpk::kSplitN * fpk::kSplitN;
       const uint64_t most = fpk::tails_above(binom(), k, 3, p - 1, -1);
       const int need = (int)std::min<uint64_t>((std::max<uint64_t>(most, fpk::tails_above(binom(), k, 2, p - 1, -1)) +
                                                 fpk::kSplitN - 1) / fpk::kSplitN * fpk::kSplitN, 1u << 20);
       P->split_cap = std::min(cap, need);
       P->split_k = K;
-      P->split = cap >= 4 * fpk::kSplitN;
+      P->split = cap >= 4 * fpk::kSplitN && fpk::split_smem(k, p, P->rwpad, P->split_cap, K) <= kSplitSmemMax;
     }
   }
   // The g = 1 passes are the rows of the Gamma_j themselves: their least
@@ -744,63 +744,92 @@ void plan_tasks(Prepared *P, int ctas, int fixed_pl, int min_steps, bool spread_
 }
 
 int split_smem_bytes(const Prepared &P) {
-  // at least half of an SM's shared memory, so that a second such CTA, which
+  // more than half of an SM's shared memory, so that a second such CTA, which
   // would wait for the first one's tensor memory, never becomes resident
   return std::max(fpk::split_smem(P.k, P.p, P.rwpad, P.split_cap, P.split_k), 120 * 1024);
 }
 
 namespace {
 
-// Issue slots of the tensor-core kernel (per warp scheduler, one warpgroup
-// at work on it): a stem's step and class values, the start of a lane's run
-// of stems, one tile of results, and the build of a block of n tails.
-constexpr double kStemSlots = 150, kRunSlots = 400, kTileSlots = 85;
-inline double build_slots(double n) { return 1000 + 0.9 * n; }
-constexpr double kTaskSlots = 5000;        // least work of a task, so that claims stay a small part
+// Clocks of an SM (its four warpgroups at work) for the parts of a split
+// pass, from traced searches: a stem step of 128 lanes, one tile of results
+// (the tensor pipe's time, or the warps' for short rows), the build of a
+// block of n tails, the start of a task's lanes.
+constexpr double kStepClocks = 500, kStartClocks = 1500;
+inline double tile_clocks(int K) { return std::max(150.0, 1.5 * K); }
+inline double build_clocks(double n) { return 2500 + 2.2 * n; }
+constexpr double kTaskClocks = 6000;         // least work of a task
 constexpr uint64_t kDirectCombos = 1 << 19;  // stem-tail pairs of a pass up to which every weight is computed exactly
 
-// Stems of pass level g with tails of t rows whose largest row is below z.
-uint64_t stems_below(const Prepared &P, int z, int l, uint64_t ncl) { return l > 0 ? binom().c[z][l] * ncl : 1; }
-
-struct SplitCost {
-  double slots = 0;  // of all warpgroups
-  int blocks = 0;
+// One way to cut a code's tails: t rows, blocks of nb.  It depends on the
+// code's shape only, so it is worked out once for all passes.
+struct TailCut {
+  struct Block {
+    uint32_t n;        // tails
+    int zhi;           // z of the first
+    uint32_t tiles;    // whole block
+    int at;            // tiles above q: tiles_at[at + q] for q < zhi, or -1: take all as `tiles`
+  };
+  int t = 0;
+  uint32_t nb = 0;
+  std::vector<Block> blocks;
+  std::vector<uint32_t> tiles_at;
 };
-// Work of a pass with tails of t rows in blocks of nb.
-SplitCost split_cost(const Prepared &P, int g, int t, uint32_t nb, uint64_t ncl) {
-  const int k = P.k, b = P.p - 1, l = g - t;
+
+TailCut cut_tails(const Prepared &P, int t, uint32_t cap) {
+  const int k = P.k, b = P.p - 1;
+  const uint32_t N = fpk::kSplitN;
   const uint32_t etot = fpk::tails_above(binom(), k, t, b, -1);
-  SplitCost c;
-  for (uint32_t first = 0; first < etot; first += nb) {
-    ++c.blocks;
-    const uint32_t n = std::min(nb, etot - first);
-    const int m = fpk::comb_floor(binom(), t - 1, k - 1, t, fpk::tail_coefs(t, b), first);
-    const int zhi = k - 1 - m;
-    if (l == 0) {
-      c.slots += kRunSlots + kTileSlots * ((n + fpk::kSplitN - 1) / fpk::kSplitN);
-      continue;
+  TailCut c;
+  c.t = t;
+  const uint32_t nblk = (etot + cap - 1) / cap;
+  if (nblk > 255) return c;  // the run's field
+  c.nb = ((etot + nblk - 1) / nblk + N - 1) / N * N;
+  for (uint32_t first = 0; first < etot; first += c.nb) {
+    TailCut::Block x;
+    x.n = std::min(c.nb, etot - first);
+    x.zhi = k - 1 - fpk::comb_floor(binom(), t - 1, k - 1, t, fpk::tail_coefs(t, b), first);
+    x.tiles = (x.n + N - 1) / N;
+    x.at = -1;
+    if (t == 2 || first == 0) {  // later blocks of three rows hold a few values of z: every stem meets most of them
+      x.at = (int)c.tiles_at.size();
+      for (int q = 0; q < x.zhi; ++q)
+        c.tiles_at.push_back((std::min(x.n, fpk::tails_above(binom(), k, t, b, q) - first) + N - 1) / N);
     }
-    if (t == 3) {  // a few values of z to a block: every stem meets most of it
-      c.slots += (double)stems_below(P, zhi, l, ncl) / 128 * (kStemSlots + kTileSlots * (double)((n + fpk::kSplitN - 1) / fpk::kSplitN));
-      continue;
-    }
-    for (int q = l - 1; q < zhi; ++q) {
-      const uint32_t e = std::min(n, fpk::tails_above(binom(), k, t, b, q) - first);
-      c.slots += (double)(binom().c[q][l - 1] * ncl) / 128 * (kStemSlots + kTileSlots * (double)((e + fpk::kSplitN - 1) / fpk::kSplitN));
-    }
+    c.blocks.push_back(x);
   }
   return c;
+}
+
+// Clocks of all SMs for a pass with stems of l rows.
+double cut_clocks(const TailCut &c, int l, uint64_t ncl, double tile) {
+  double sum = 0;
+  for (const auto &x : c.blocks) {
+    if (l == 0) {
+      sum += kStepClocks + tile * x.tiles;
+    } else if (x.at < 0) {
+      sum += (double)(binom().c[x.zhi][l] * ncl) * (kStepClocks + tile * x.tiles) / 128;
+    } else {
+      double s = 0;
+      for (int q = l - 1; q < x.zhi; ++q) s += (double)binom().c[q][l - 1] * (kStepClocks + tile * c.tiles_at[x.at + q]);
+      sum += s * (double)ncl / 128;
+    }
+  }
+  return sum;
 }
 
 }  // namespace
 
 // Every pass with g >= 2 gets its tail length, block size and runs of
-// tasks.  Tails of three rows serve a stem more entries (their blocks are
-// full but for the stem's step), tails of two need fewer tables; the
-// cheaper of the two by the slots above.
+// tasks.  Tails of three rows serve a stem more entries, tails of two need
+// fewer tables; the cheaper of the two by the clocks above.
 void plan_split(Prepared *P, int ctas) {
   const double C = std::max(1, ctas);
   const int k = P->k, b = P->p - 1;
+  const double tile = tile_clocks(P->split_k);
+  const uint32_t cap = (uint32_t)P->split_cap;
+  const TailCut cuts[3] = {cut_tails(*P, 2, cap), cut_tails(*P, 3, cap),
+                           cut_tails(*P, 3, std::max<uint32_t>(fpk::kSplitN, cap / 2 / fpk::kSplitN * fpk::kSplitN))};
   P->split_segs.clear();
   for (auto &d : P->passes) {
     d.phases = 0;
@@ -827,42 +856,37 @@ void plan_split(Prepared *P, int ctas) {
     int t = 2;
     uint32_t nb = 0;
     double total = 0;
+    const TailCut *cut = nullptr;
     const uint64_t combos = g == 2 ? d.size : d.size / 2;
     if (combos <= kDirectCombos) {
       d.direct = 1;
       nb = fpk::tails_above(binom(), k, 2, b, -1);
     } else {
       double best = 0;
-      for (int tt = 2; tt <= 3; ++tt) {
-        if (tt == 3 && g < 4) break;
-        const uint32_t etot = fpk::tails_above(binom(), k, tt, b, -1);
-        for (int half = 0; half < (tt == 3 ? 2 : 1); ++half) {
-          const uint32_t cap = std::max<uint32_t>(fpk::kSplitN, (uint32_t)(P->split_cap >> half) / fpk::kSplitN * fpk::kSplitN);
-          const uint32_t nblk = (etot + cap - 1) / cap;
-          if (nblk > 255) continue;  // the run's field
-          const uint32_t size = ((etot + nblk - 1) / nblk + fpk::kSplitN - 1) / fpk::kSplitN * fpk::kSplitN;
-          const SplitCost c = split_cost(*P, g, tt, size, ncl_of(g - tt));
-          const double tasks = std::max<double>(c.blocks, std::min(C, c.slots / kTaskSlots));
-          const double cost = c.slots / C + build_slots(size) * std::max(1.0, tasks / C);
-          if (nb == 0 || cost < best) {
-            best = cost;
-            t = tt;
-            nb = size;
-            total = c.slots;
-          }
+      for (const TailCut &c : cuts) {
+        if (c.blocks.empty() || (c.t == 3 && g < 4)) continue;
+        const double clocks = cut_clocks(c, g - c.t, ncl_of(g - c.t), tile);
+        // a CTA takes at least one task, and builds a table for most of the tasks of a pass with several blocks
+        const double tasks = std::max<double>((double)c.blocks.size(), std::min(C, clocks / kTaskClocks));
+        const double cost = clocks / C + (build_clocks(c.nb) + kStartClocks) * std::max(1.0, tasks / C);
+        if (!cut || cost < best) {
+          best = cost;
+          cut = &c;
+          total = clocks;
         }
       }
+      t = cut->t;
+      nb = cut->nb;
     }
     const int l = g - t;
     d.tail_rows = (uint8_t)t;
     d.block = nb;
     d.ncl = ncl_of(l);
-    const uint32_t etot = fpk::tails_above(binom(), k, t, b, -1);
     uint32_t tasks = 0;
     auto add = [&](uint32_t item0, uint32_t item1, uint64_t per, uint32_t block, int zhi) {
       if (item0 >= item1) return;
       fpk::SplitSeg s{};
-      per = std::min<uint64_t>(std::max<uint64_t>(per, 1), 65535);
+      per = std::min<uint64_t>(std::max<uint64_t>(per, 1), 65532);
       tasks += (uint32_t)((item1 - item0 + per - 1) / per);
       s.task_end = tasks;
       s.item0 = item0;
@@ -873,51 +897,54 @@ void plan_split(Prepared *P, int ctas) {
       P->split_segs.push_back(s);
     };
     if (d.direct) {
+      // runs of stems with about the same number of tails, as many to a task
+      // as give every warpgroup of the grid the same work
       d.esplit = g == 2 ? 2 : 0;
-      const uint32_t items = (uint32_t)(stems_below(*P, k - 2, l, d.ncl) << d.esplit);
-      add(0, items, std::max<uint64_t>(4, (uint64_t)((items + C - 1) / C)), 0, k - 2);
+      auto stem_clocks = [&](int q) {
+        return 400.0 + 800.0 * (double)((fpk::tails_above(binom(), k, t, b, q) + fpk::kSplitGroup - 1) / fpk::kSplitGroup);
+      };
+      double work = 0;
+      for (int q = std::max(l - 1, 0); l > 0 && q < k - 2; ++q) work += (double)(binom().c[q][l - 1] * d.ncl) * stem_clocks(q);
+      const uint32_t items = (uint32_t)(l > 0 ? binom().c[k - 2][l] * d.ncl : 1);
+      // the passes of one level run side by side, one per information set
+      const double target = std::max(3000.0, work * std::min(P->m, 4) / (4 * C));
+      uint32_t at = 0;
+      for (int q = std::max(l - 1, 0); at < items;) {
+        const double c = stem_clocks(l > 0 ? q : -1);
+        int q1 = q + 1;
+        while (l > 0 && q1 < k - 2 && stem_clocks(q1) * 1.3 >= c) ++q1;
+        const uint32_t end = l > 0 && q1 < k - 2 ? (uint32_t)(binom().c[q1][l] * d.ncl) : items;
+        add(at, end, l > 0 ? 4 * std::max<uint64_t>(1, (uint64_t)(target / c)) : 1, 0, k - 2);
+        at = std::max(at, end);
+        q = q1;
+      }
     } else {
-      // stems per lane: long runs share the start of a lane, as long as the
-      // grid's warpgroups get eight items each
-      uint64_t stems = 0;
-      for (uint32_t first = 0, blk = 0; first < etot; first += nb, ++blk)
-        stems += stems_below(*P, k - 1 - fpk::comb_floor(binom(), t - 1, k - 1, t, fpk::tail_coefs(t, b), first), l, d.ncl);
-      uint32_t T = 1;
-      while (T < 32 && stems / (128 * 2 * T) >= (uint64_t)(8 * 4 * C)) T *= 2;
-      while (stems / (128ull * T) >= (1ull << 26)) T *= 2;  // items fit 32 bits with their slices
-      const uint32_t tiles_max = (std::min(nb, etot) + fpk::kSplitN - 1) / fpk::kSplitN;
-      int es = 0;
-      while (es < 4 && (stems / 128 << es) < (uint64_t)(4 * C) && (tiles_max >> es) >= 4) ++es;
-      d.unit = T;
-      d.esplit = (uint8_t)es;
+      // a task of least size: 4 units with all warpgroups on their own, or
+      // 2 or 1 with their tails split
+      const double unit_max = kStepClocks + tile * cut->blocks[0].tiles;
+      const double target0 = std::max(kTaskClocks, std::min(total / C, 4 * kTaskClocks));
+      d.esplit = 4 * unit_max <= 1.5 * target0 ? 0 : 2 * unit_max <= 1.5 * target0 ? 1 : 2;
+      const uint64_t parts = 4u >> d.esplit;
       double rem = total;
-      for (uint32_t first = 0, blk = 0; first < etot; first += nb, ++blk) {
-        const uint32_t n = std::min(nb, etot - first);
-        const int zhi = k - 1 - fpk::comb_floor(binom(), t - 1, k - 1, t, fpk::tail_coefs(t, b), first);
-        const uint64_t ns = stems_below(*P, zhi, l, d.ncl);
-        const uint32_t items = (uint32_t)(((ns + 128ull * T - 1) / (128ull * T)) << es);
-        // runs of items whose first stem meets the same number of tiles
+      for (uint32_t blk = 0; blk < cut->blocks.size(); ++blk) {
+        const TailCut::Block &x = cut->blocks[blk];
+        const uint64_t ns = l > 0 ? binom().c[x.zhi][l] * d.ncl : 1;
+        const uint32_t units = (uint32_t)((ns + 127) / 128);
+        auto tiles_at = [&](int q) { return l > 0 && x.at >= 0 ? cut->tiles_at[x.at + q] : x.tiles; };
+        // runs of units whose first stem meets about the same number of tiles
         uint32_t at = 0;
-        int q = std::max(l - 1, 0);
-        while (at < items) {
-          const uint32_t e = l > 0 ? std::min(n, fpk::tails_above(binom(), k, t, b, q) - first) : n;
-          const uint32_t tiles = (e + fpk::kSplitN - 1) / fpk::kSplitN;
+        for (int q = std::max(l - 1, 0); at < units;) {
+          const uint32_t tiles = tiles_at(q);
           int q1 = q + 1;
-          if (t == 3) q1 = zhi;
-          while (l > 0 && q1 < zhi &&
-                 (std::min(n, fpk::tails_above(binom(), k, t, b, q1) - first) + fpk::kSplitN - 1) / fpk::kSplitN == tiles)
-            ++q1;
-          uint32_t end = items;
-          if (l > 0 && q1 < zhi) end = std::min<uint32_t>(items, (uint32_t)((binom().c[q1][l] * d.ncl / (128ull * T)) << es));
+          while (l > 0 && q1 < x.zhi && tiles_at(q1) * 8 >= tiles * 7) ++q1;
+          uint32_t end = units;
+          if (l > 0 && q1 < x.zhi) end = std::min<uint32_t>(units, (uint32_t)(binom().c[q1][l] * d.ncl / 128));
           if (end > at) {
-            const double per_item = kRunSlots + T * (kStemSlots + kTileSlots * std::max(1.0, (double)tiles / (1 << es)));
-            const double target = std::max(kTaskSlots, rem / (2 * C));
-            uint64_t per = (uint64_t)(target / per_item + 0.5);
-            if (per > 4) per = per / 4 * 4;  // the four warpgroups of a CTA share a task's items
-            if (per < 4) per = 4;
-            add(at, end, per, blk, zhi);
-            rem -= per_item * (end - at);
-            if (rem < 0) rem = 0;
+            const double unit = kStepClocks + tile * tiles;
+            const double target = std::max(kTaskClocks, rem / (2 * C));
+            const uint64_t per = (uint64_t)(target / (unit * (double)parts) + 0.5) * parts;
+            add(at, end, std::max<uint64_t>(per, parts), blk, x.zhi);
+            rem = std::max(0.0, rem - unit * (end - at));
             at = end;
           }
           q = q1;
@@ -1249,35 +1276,34 @@ int fpcode_test_key_coefficients(const fpcode_prepared *prep, uint64_t key, int 
 
 extern "C++" {
 namespace {
-// The codewords of items [lo, hi) of one tail block, as the kernel walks
-// them (lanes in order, steps, tiles of the item's slice), as packed keys
-// of weight 0.
+// The codewords of units [lo, hi) of one tail block, as the kernel walks
+// them (warpgroups and lanes in order, steps, tiles of the slice), as packed
+// keys of weight 0.
 template <int DB, class F>
 void split_walk(const fph::Prepared &P, const fpk::PassDesc &d, int pass, uint64_t lo, uint64_t hi, uint32_t block,
                 int zhi, F emit) {
   const fpenum::Binom &B = fph::binom();
   const int k = P.k, b = P.p - 1, g = d.g, t = d.tail_rows, l = g - t;
   const uint32_t etot = fpk::tails_above(B, k, t, b, -1), first = block * d.block;
-  const uint32_t nb = std::min(d.block, etot - first), slices = 1u << d.esplit;
+  const uint32_t nb = std::min(d.block, etot - first), slices = 1u << d.esplit, parts = 4u >> d.esplit;
   const uint64_t ns = l > 0 ? B(zhi, l) * d.ncl : 1;
-  const uint32_t T = d.direct ? 1 : d.unit, lanes = d.direct ? 1 : fpk::kSplitGroup;
-  const uint32_t tile = d.direct ? fpk::kSplitGroup : fpk::kSplitN;
-  for (uint64_t item = lo; item < hi; ++item) {
-    const uint64_t J0 = (item >> d.esplit) * lanes * T;
-    const uint32_t slice = (uint32_t)item & (slices - 1);
-    if (J0 >= ns) continue;
+  const uint32_t lanes = d.direct ? 1 : fpk::kSplitGroup, tile = d.direct ? fpk::kSplitGroup : fpk::kSplitN;
+  const uint64_t share = (hi - lo + parts - 1) / parts;
+  for (uint32_t grp = 0; grp < 4; ++grp) {
+    const uint32_t part = grp >> d.esplit, slice = grp & (slices - 1);
+    const uint64_t u0 = std::min(lo + part * share, hi), steps = std::min(u0 + share, hi) - u0, J0 = u0 * lanes;
+    if (steps == 0 || J0 >= ns) continue;
     const int q0 = l > 0 ? fpk::comb_floor(B, l - 1, k - t - 1, l, d.ncl, J0) : -1;
     const uint32_t tiles = (std::min(nb, fpk::tails_above(B, k, t, b, q0) - first) + tile - 1) / tile;
     for (uint32_t lane = 0; lane < lanes; ++lane) {
-      const uint64_t J = J0 + (uint64_t)lane * T;
-      const uint32_t nst = J < ns ? (uint32_t)std::min<uint64_t>(T, ns - J) : 0;
+      const uint64_t J = J0 + lane * steps, nst = J < ns ? std::min(steps, ns - J) : 0;
       fpenum::Prefix pf{-1, 0, 0, 0};
       uint64_t ci = 0, nq = 1;
       if (nst && l > 0) {
         pf = fpk::stem_unrank<DB>(B, J, k, t, l, b, d.ncl, &ci);
         nq = B(pf.m, l - 1);
       }
-      for (uint32_t i = 0; i < nst; ++i) {
+      for (uint64_t i = 0; i < nst; ++i) {
         for (uint32_t c = slice; c < tiles; c += slices)
           for (uint32_t e = c * tile; e < std::min((c + 1) * tile, nb); ++e) {
             const fpk::Tail a = fpk::tail_unpack(fpk::tail_pack(fpk::tail_unrank(B, first + e, k, t, b)));
@@ -1334,19 +1360,18 @@ int64_t fpcode_test_split_pass(fpcode_prepared *prep, int pass, int ctas, int ta
     return n;
   }
   const int l = d.g - tail_rows;
-  if (tail_rows < 2 || tail_rows > 3 || l < 0 || block < 1 || unit < 1 || esplit < 0) return -1;
+  if (tail_rows < 2 || tail_rows > 3 || l < 0 || block < 1 || unit < 1 || esplit < 0 || esplit > 2) return -1;
   d.direct = 0;
   d.tail_rows = (uint8_t)tail_rows;
   d.block = (uint32_t)block;
-  d.unit = (uint32_t)unit;
   d.esplit = (uint8_t)esplit;
   d.ncl = l > 0 ? (uint64_t)(b / 2) : 1;
   for (int i = 1; i < l; ++i) d.ncl *= (uint64_t)b;
   const uint32_t etot = fpk::tails_above(fph::binom(), k, tail_rows, b, -1);
   for (uint32_t first = 0, blk = 0; first < etot; first += (uint32_t)block, ++blk) {
     const int zhi = fpk::tail_unrank(fph::binom(), first, k, tail_rows, b).z;
-    const uint64_t ns = l > 0 ? fph::binom()(zhi, l) * d.ncl : 1;
-    walk(0, ((ns + 128ull * unit - 1) / (128ull * unit)) << esplit, blk, zhi);
+    const uint64_t units = ((l > 0 ? fph::binom()(zhi, l) * d.ncl : 1) + 127) / 128;
+    for (uint64_t u = 0; u < units; u += (uint64_t)unit) walk(u, std::min<uint64_t>(u + unit, units), blk, zhi);
   }
   return n;
 }

@@ -24,10 +24,11 @@
 
 namespace fpk {
 
-// One run of tasks of a split pass: items [item0, item1) of one tail block,
-// `per` to a task.  An item is one run of PassDesc.unit stems for each of
-// 128 lanes (tensor-core passes) or one stem (direct passes), over one of
-// 1 << esplit interleaved slices of the block's tails.
+// One run of tasks of a split pass: units [item0, item1) of one tail block,
+// `per` to a task.  A unit is 128 stems (tensor-core passes) or one stem
+// (direct passes).  The four warpgroups of a CTA share a task's units
+// evenly, or (esplit 1, 2) half or all of them share the same units and
+// take interleaved slices of the block's tails.
 struct SplitSeg {
   uint32_t task_end;  // tasks of the pass up to the end of this run
   uint32_t item0, item1;
@@ -37,7 +38,7 @@ struct SplitSeg {
 };
 static_assert(sizeof(SplitSeg) == 16, "SplitSeg layout");
 
-// Items [lo, hi) of task t of a split pass whose runs are seg[0 .. nseg);
+// Units [lo, hi) of task t of a split pass whose runs are seg[0 .. nseg);
 // returns the run.
 FPK_HD SplitSeg split_task(const SplitSeg *seg, int nseg, uint64_t t, uint64_t *lo, uint64_t *hi) {
   int a = 0, z = nseg - 1;
@@ -54,7 +55,7 @@ FPK_HD SplitSeg split_task(const SplitSeg *seg, int nseg, uint64_t t, uint64_t *
   return g;
 }
 
-constexpr int kSplitThreads = 512;  // threads per CTA of the tensor-core kernel
+constexpr int kSplitThreads = 512;  // working threads per CTA of the tensor-core kernel (one more warp claims)
 constexpr int kSplitGroup = 128;    // lanes per warpgroup: rows of one accumulator tile
 constexpr int kSplitN = 96;         // tails per accumulator tile
 
@@ -289,22 +290,24 @@ FPK_HD int class_vals(int p) { return p == 3 ? 1 : 3; }
 // K (values per row, a multiple of 32) and positions compared for n - k = N
 // redundant symbols; K = 0: the code does not fit.  Four values of the last
 // word hold the threshold and the padding mark.  A comparison of fewer
-// positions is a weaker bound; up to a tenth of them are left out where
-// that saves 32 values a row.
+// positions is a weaker bound: one position in 32 is left out where that
+// saves 32 values a row, no more (F_7 [52,19] at 30 of 33 positions: 43 % of
+// a warp's tiles held a candidate, and their exact checks cost more than the
+// shorter rows saved).
 FPK_HD int split_k(int p, int N, int *nu) {
   const int v = class_vals(p);
   int K = (v * N + 4 + 31) / 32 * 32;
   *nu = N;
   const int fit = (K - 32 - 4) / v;  // positions that 32 values fewer hold
-  if (K > 32 && fit < N && (N - fit) * 10 <= N) {
+  if (K > 32 && fit < N && (N - fit) * 32 <= N) {
     K -= 32;
     *nu = fit;
   }
   return K <= 128 ? K : 0;
 }
 
-// Shared memory of a CTA: binomial columns, one set's multiples, the packed
-// tails of a block, then (128-byte aligned) their K class values each.
+// Shared memory of a CTA: the binomial columns, one set's multiples, the
+// packed tails of a block, then (128-byte aligned) their K class values.
 constexpr int kSplitBinomBytes = fpenum::kBinomCols * (fpenum::kMaxK + 1) * 8;
 FPK_HD int split_mult_words(int k, int p, int rwpad) { return k * (p - 1) * rwpad; }
 FPK_HD int split_off_tails(int k, int p, int rwpad) {
@@ -313,6 +316,10 @@ FPK_HD int split_off_tails(int k, int p, int rwpad) {
 FPK_HD int split_off_table(int k, int p, int rwpad, int cap) {
   return (split_off_tails(k, p, rwpad) + cap * 4 + 127) / 128 * 128;
 }
-FPK_HD int split_smem(int k, int p, int rwpad, int cap, int K) { return split_off_table(k, p, rwpad, cap) + cap * K; }
+FPK_HD int split_smem(int k, int p, int rwpad, int cap, int K) {
+  const int block = split_off_table(k, p, rwpad, cap) + cap * K;
+  const int direct = split_off_tails(k, p, rwpad) + (p - 1) * (k * (k - 1) / 2) * 4;  // packed tails of two rows alone
+  return block > direct ? block : direct;
+}
 
 }  // namespace fpk

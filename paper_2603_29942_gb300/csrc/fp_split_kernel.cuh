@@ -190,6 +190,7 @@ __device__ __noinline__ void build_tails(uint32_t *tails, char *table, const uin
   const uint32_t rows = with_table ? (n + kSplitN - 1) / kSplitN * kSplitN : n;
   const uint32_t run = ((rows + kSplitThreads - 1) / kSplitThreads) | 1u;
   const uint32_t e0 = threadIdx.x * run, e1 = min(e0 + run, rows);
+  const int vals = nu * ClassCode<P>::kVals;
   if (e0 >= e1) return;
   Tail a{};
   uint32_t part[RW];
@@ -214,16 +215,18 @@ __device__ __noinline__ void build_tails(uint32_t *tails, char *table, const uin
     }
     if (with_table) {
       char *row = table + (size_t)(e >> 3) * (8 * K) + (e & 7) * 16;
-      const int vals = e < n ? nu * ClassCode<P>::kVals : 0;
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
         if (32 * s >= K) break;
-        uint32_t w[8];
-        class_bytes(o[s], w);
+        uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+        const int left = vals - 32 * s;  // the same for all tails
+        if (e < n && left > 0) {
+          class_bytes(o[s], w);
+          if (left < 32) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int left = vals - (32 * s + 4 * i);
-          w[i] = left >= 4 ? w[i] : left > 0 ? w[i] & ((1u << (8 * left)) - 1u) : 0u;
+            for (int i = 0; i < 8; ++i)
+              w[i] = left >= 4 * i + 4 ? w[i] : left > 4 * i ? w[i] & ((1u << (8 * (left - 4 * i))) - 1u) : 0u;
+          }
         }
         if (32 * (s + 1) == K) w[7] = e < n ? kTailMarks : kTailPadding;
         *reinterpret_cast<uint4 *>(row + s * 256) = make_uint4(w[0], w[1], w[2], w[3]);
@@ -238,13 +241,27 @@ struct SplitQueue {
   uint32_t item[64];  // fewer than 32 left over, then at most one per lane
 };
 
-// What the lanes of a CTA share while they run a task.
+// A task as the scheduler warp hands it to the warpgroups.
+struct SplitTask {
+  Claim cl;
+  PassDesc pd;
+  int cmd;                   // kCmdRun or kCmdExit
+  int stage, build;          // stage the set's multiples; build its tail block: 1 packed tails, 2 also the B operand
+  int drop;                  // the code finished before the task began
+  unsigned long long count;  // codewords evaluated
+};
+
+// What the threads of a CTA share.
 struct SplitShared {
-  uint32_t next;                  // items handed out
-  uint32_t item[kSplitGroups];    // a warpgroup's item (~0: none left)
-  int32_t stop[kSplitGroups][2];  // by the parity of the step: the code has finished, the warpgroup drops the rest of
-                                  // its item (two, since the first warp may be a step ahead of the last)
+  int32_t stop[kSplitGroups][2];  // by the parity of the product: the code has finished, the warpgroup drops the rest
+                                  // of its task (two, since the first warp may be a product ahead of the last)
+  unsigned long long best_key;    // the code's best key (inverted) and finished flag, as the scheduler last read them
+  int32_t finished;
   SplitQueue queue[kSplitWarps];
+  SplitTask task[2];              // the one that runs and the next one
+  // mbarriers: of each task buffer, full (1 arrival), near its end (one per
+  // warpgroup) and done (one per warp); of each warpgroup, its products
+  unsigned long long full[2], near[2], done[2], product[kSplitGroups];
 };
 
 // The stem a lane holds: its exact sum, its rows and coefficients.
@@ -323,12 +340,16 @@ __device__ __noinline__ uint64_t hit_key(const fpenum::BinomCols B, bool pair, i
   return best;
 }
 
-// One task of a pass with g >= 2: items [lo, hi) of one tail block.
+// One task of a pass with g >= 2: units [ulo, uhi) of one tail block, a
+// unit being 128 stems (tensor-core passes) or one stem (direct passes).
+// Every warpgroup takes an equal run of them (esplit 0), or a run and one of
+// 2 or 4 interleaved slices of the tails, so nothing is handed out inside a
+// task; `near` is told when its last step begins.
 template <int P, int R, int W>
 __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &cl, const uint32_t *mult,
                            const uint32_t *tails, uint32_t table, uint32_t tmem, uint32_t mbar, uint32_t &parity,
-                           const fpenum::BinomCols &B, SplitShared &sh, SlotState *st, SlotAux *ax, CtlDyn *cd,
-                           unsigned long long &count) {
+                           uint32_t near, const fpenum::BinomCols &B, SplitShared &sh, SlotState *st, SlotAux *ax,
+                           CtlDyn *cd, unsigned long long &count) {
   constexpr int DB = P == 3 ? 1 : 4, RW = R * W, b = P - 1;
   constexpr unsigned FULL = 0xffffffffu;
   const int k = sd.k, g = pd.g, t = pd.tail_rows, l = g - t, pass = cl.pass;
@@ -341,23 +362,28 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
   const uint64_t ns = l > 0 ? B(cl.zhi, l) * ncl : 1ull;
   const int K = sd.split_k, nu = sd.split_nu;
   const unsigned long long cpe = l > 0 ? 2ull : 1ull;  // codewords per stem and tail
-  const uint32_t nitems = (uint32_t)(cl.uhi - cl.ulo);
+  // the warpgroup's units [u0, u0 + steps) and its slice of the tails
+  const uint32_t parts = (uint32_t)kSplitGroups >> pd.esplit, part = (uint32_t)grp >> pd.esplit;
+  const uint32_t slices = 1u << pd.esplit, slice = (uint32_t)grp & (slices - 1u);
+  const uint32_t share = ((uint32_t)(cl.uhi - cl.ulo) + parts - 1) / parts;
+  const uint64_t u0 = min(cl.ulo + (uint64_t)part * share, cl.uhi);
+  const uint32_t steps = (uint32_t)(min(u0 + share, cl.uhi) - u0);
+  auto nearly = [&]() {
+    if (row == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(near) : "memory");
+  };
   int thr = cl.U - g + 1;  // record weights <= U: redundant weight < U - g + 1
   SplitQueue &wq = sh.queue[warp];
 
-  // up to date with the records of the other warps: lane 0 reads, the value is taken up a step later
-  int pfin = 0;
-  unsigned long long pkey = 0;
-  auto poll = [&]() {
-    if (lane == 0) {
-      pfin = ld_vol(&st->finished);
-      pkey = ld_vol(&st->best_key);
-    }
-  };
+  // Up to date with the records of other warps and CTAs: the scheduler warp
+  // keeps reading the best key and the finished flag into shared memory.  (A
+  // load by each warp cost it 2 us a step: the value's first use waits for
+  // the L2, which serves the one line to every warp of the grid.)
   auto take_up = [&]() {
-    const uint64_t key = ~(uint64_t)__shfl_sync(FULL, pkey, 0);
+    const uint64_t key = ~(uint64_t)*(volatile unsigned long long *)&sh.best_key;
     if (key != kNoKey) thr = min(thr, (int)key_weight(key) - g + 1);
+    thr = (int)__reduce_min_sync(FULL, (unsigned)max(thr, 0));  // one value for the warp
   };
+  auto finished = [&]() { return *(volatile int32_t *)&sh.finished; };
   auto note = [&](uint64_t best) {  // the warp's best key, if any lane has one
     if (__any_sync(FULL, best != kNoKey)) {
 #pragma unroll
@@ -366,18 +392,6 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
       thr = min(thr, (int)key_weight(best) - g + 1);
     }
   };
-  // the next item of the warpgroup (every lane gets it)
-  auto grab = [&]() -> uint32_t {
-    if (row == 0) {
-      const uint32_t i = pfin ? ~0u : atomicAdd(&sh.next, 1u);
-      sh.item[grp] = i < nitems ? i : ~0u;
-    }
-    group_sync(1 + grp);
-    const uint32_t i = *(volatile uint32_t *)&sh.item[grp];
-    group_sync(1 + grp);
-    return i;
-  };
-
   Stem<RW> x;
 #pragma unroll
   for (int q = 0; q < RW; ++q) x.s[q] = 0;
@@ -387,21 +401,16 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
   x.qrows = 0;
 
   if (pd.direct) {
-    // few codewords: one stem per item, its tails over the 128 lanes, every
-    // weight exact (no table; before the first records most bounds would
+    // few codewords: one stem per warpgroup at a time, its tails over the 128
+    // lanes, every weight exact (no table; before the first records most bounds would
     // pass the threshold anyway)
-    poll();
-    for (;;) {
-      const uint32_t it = grab();
-      if (it == ~0u) return;
-      const uint64_t item = cl.ulo + it;
-      const uint64_t J = item >> pd.esplit;
-      const uint32_t slice = (uint32_t)item & ((1u << pd.esplit) - 1u);
-      if (l > 0) stem_start<P, R, W, DB>(x, mult, B, J, k, t, l, ncl);
+    nearly();
+    if (l > 0 && steps) stem_start<P, R, W, DB>(x, mult, B, u0, k, t, l, ncl);
+    for (uint32_t i = 0; i < steps && !finished(); ++i) {
+      if (l > 0 && i) stem_next<P, R, W, DB>(x, mult, B, l, ncl);
       const uint32_t E = min(nb, tails_above(B, k, t, b, x.pf.m) - first);
       take_up();
-      poll();
-      for (uint32_t e0 = slice * kSplitGroup; e0 < E; e0 += kSplitGroup << pd.esplit) {
+      for (uint32_t e0 = slice * kSplitGroup; e0 < E; e0 += kSplitGroup * slices) {
         const uint32_t e = e0 + row;
         uint64_t best = kNoKey;
         if (e < E) {
@@ -415,207 +424,236 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
         note(best);
       }
     }
+    return;
   }
 
-  const uint32_t T = pd.unit;  // stems per lane and item
   const uint32_t tA = tmem + (uint32_t)grp * (kTmemCols / kSplitGroups), tD = tA + kTmemD;
   const uint32_t my_lanes = (uint32_t)(warp & 3) << 21;  // 32 lanes a warp, in the address's upper half
   bool dead = false;
-  poll();
-  for (;;) {
-    const uint32_t it = grab();
-    if (it == ~0u) return;
-    const uint64_t item = cl.ulo + it;
-    const uint64_t run = item >> pd.esplit;
-    const uint32_t slice = (uint32_t)item & ((1u << pd.esplit) - 1u), slices = 1u << pd.esplit;
-    const uint64_t J0 = run * (uint64_t)(kSplitGroup * T), J = J0 + (uint64_t)row * T;
-    const uint32_t nst = J < ns ? (uint32_t)min((uint64_t)T, ns - J) : 0u;
-    if (l > 0 && nst) stem_start<P, R, W, DB>(x, mult, B, J, k, t, l, ncl);
-    // tails of the block above the item's first stem: as many tiles as any lane needs
-    const int q0 = l > 0 ? comb_floor(B, l - 1, k - t - 1, l, ncl, J0) : -1;
-    const uint32_t tiles = (min(nb, tails_above(B, k, t, b, q0) - first) + kSplitN - 1) / kSplitN;
-    if (slice >= tiles) continue;  // the same for the whole warpgroup
-    for (uint32_t i = 0; i < T; ++i) {
-      const bool act = i < nst;
-      take_up();
-      if (row == 0) *(volatile int32_t *)&sh.stop[grp][i & 1u] = pfin;
-      poll();
-      {
-        __syncwarp();
-        uint32_t o[4], w[8];
-        class_bits<P, R, W>(x.s, nu, o);
-        const uint32_t marks = act ? stem_marks<P>(nu, thr) : kStemNone;
+  const uint64_t J0 = u0 * kSplitGroup, J = J0 + (uint64_t)row * steps;  // a lane's run of stems
+  const uint32_t nst = J < ns ? (uint32_t)min((uint64_t)steps, ns - J) : 0u;
+  if (l > 0 && nst) stem_start<P, R, W, DB>(x, mult, B, J, k, t, l, ncl);
+  // tails of the block above the run's first stem: as many tiles as any lane needs
+  const int q0 = l > 0 && steps ? comb_floor(B, l - 1, k - t - 1, l, ncl, J0) : -1;
+  const uint32_t tiles = (min(nb, tails_above(B, k, t, b, q0) - first) + kSplitN - 1) / kSplitN;
+  if (steps == 0 || slice >= tiles) {  // the same for the whole warpgroup
+    nearly();
+    return;
+  }
+  for (uint32_t i = 0; i < steps; ++i) {
+    if (i + 1 == steps) nearly();
+    const bool act = i < nst;
+    take_up();
+    {
+      __syncwarp();
+      uint32_t o[4], w[8];
+      class_bits<P, R, W>(x.s, nu, o);
+      const uint32_t marks = act ? stem_marks<P>(nu, thr) : kStemNone;
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-          if (32 * s >= K) break;
-          class_bytes(o[s], w);
-          if (32 * (s + 1) == K) w[7] = marks;
-          tmem_store8(tA + my_lanes + 8 * s, w);
-        }
-        tmem_wait_store();
+      for (int s = 0; s < 4; ++s) {
+        if (32 * s >= K) break;
+        class_bytes(o[s], w);
+        if (32 * (s + 1) == K) w[7] = marks;
+        tmem_store8(tA + my_lanes + 8 * s, w);
       }
-      uint32_t n = 0;  // candidates in the warp's queue
-      // exact weights of `cnt` candidates from `at`: a lane takes one and fetches the owner's stem
-      auto check = [&](uint32_t at, uint32_t cnt) {
-        __syncwarp();
-        const bool have = (uint32_t)lane < cnt;
-        const uint32_t item_ = have ? wq.item[at + lane] : 0u;
-        const int src = (int)(item_ & 31u);
-        uint32_t so[RW];
-#pragma unroll
-        for (int q = 0; q < RW; ++q) so[q] = __shfl_sync(FULL, x.s[q], src);
-        const int qo = __shfl_sync(FULL, x.pf.m, src);
-        const uint32_t tl = tails[item_ >> 5];
-        const Tail a = tail_unpack(tl);
-        int wp = 1 << 20, wm = 1 << 20;
-        if (have && a.z > qo) split_weights<P, R, W>(so, a, mult, wp, wm);
-        const bool hit = wp < thr || (l > 0 && wm < thr);
-        if (__any_sync(FULL, hit)) {
-          fpenum::Prefix po;
-          po.m = qo;
-          po.qi = 0;
-          po.Q = __shfl_sync(FULL, (unsigned long long)x.pf.Q, src);
-          po.d = __shfl_sync(FULL, (unsigned long long)x.pf.d, src);
-          note(hit ? hit_key<DB>(B, pair, k, P, g, pass, wp, wm, thr, po, l, tl) : kNoKey);
-        }
-        __syncwarp();
-      };
-      // candidates among 32 results (columns col0 ..): those of sign 0
-      auto scan = [&](const uint32_t (&v)[16], uint32_t col0) {
-        uint32_t m = 0;
-#pragma unroll
-        for (int q = 0; q < 16; ++q) m = (m >> 1) | (~v[q] & 0x80008000u);
-        unsigned any;
-        while ((any = __ballot_sync(FULL, m != 0)) != 0) {
-          if (m) {
-            const int bit = fpenum::ctz32(m);
-            m &= m - 1;
-            wq.item[n + __popc(any & ((1u << lane) - 1u))] =
-                (col0 + 2u * (uint32_t)(bit & 15) + (uint32_t)(bit >> 4)) << 5 | (uint32_t)lane;
-          }
-          n += __popc(any);
-          if (n >= 32) {
-            n -= 32;
-            check(n, 32);
-          }
-        }
-      };
-      for (uint32_t c = slice; c < tiles; c += slices) {
-        tc_before_sync();
-        if ((warp & 3) == 0) {
-          group_sync(1 + grp);
-          tc_after_sync();
-          if (elect_one()) {
-            const uint64_t d0 = tile_desc(table + c * (uint32_t)(kSplitN * K), (uint32_t)K);
-            mma_step<false>(tD, tA, d0, kSplitIdesc);
-            if (K > 32) mma_step<true>(tD, tA + 8, d0 + 16, kSplitIdesc);
-            if (K > 64) mma_step<true>(tD, tA + 16, d0 + 32, kSplitIdesc);
-            if (K > 96) mma_step<true>(tD, tA + 24, d0 + 48, kSplitIdesc);
-            mma_commit(mbar);
-          }
-          __syncwarp();
-        } else {
-          group_arrive(1 + grp);
-        }
-        if (!dead && !mbar_wait(mbar, parity)) {
-          dead = true;  // never seen: reported as a timeout, and the rest of the launch drains without results
-          atomicExch(&cd->err, 1);
-        }
-        __syncwarp();
-        parity ^= 1u;
-        tc_after_sync();
-        uint32_t v0[16], v1[16], v2[16];
-        tmem_load16(tD + my_lanes, v0);
-        tmem_load16(tD + my_lanes + 32, v1);
-        tmem_load16(tD + my_lanes + 64, v2);
-        tmem_wait_load(v0, v1, v2);
-        uint32_t a0 = ~0u, a1 = ~0u, a2 = ~0u;
-#pragma unroll
-        for (int q = 0; q < 16; q += 2) {
-          a0 = and3(a0, v0[q], v0[q + 1]);
-          a1 = and3(a1, v1[q], v1[q + 1]);
-          a2 = and3(a2, v2[q], v2[q + 1]);
-        }
-        if (__any_sync(FULL, (~and3(a0, a1, a2) & 0x80008000u) != 0)) {
-          if (__any_sync(FULL, (~a0 & 0x80008000u) != 0)) scan(v0, c * kSplitN);
-          if (__any_sync(FULL, (~a1 & 0x80008000u) != 0)) scan(v1, c * kSplitN + 32);
-          if (__any_sync(FULL, (~a2 & 0x80008000u) != 0)) scan(v2, c * kSplitN + 64);
-        }
-      }
-      const int stop = *(volatile int32_t *)&sh.stop[grp][i & 1u];
-      if (n) check(0, n);
-      if (act) {
-        // this lane's tails, in this item's tiles
-        const uint32_t above = tails_above(B, k, t, b, x.pf.m);
-        const uint32_t E = above > first ? min(nb, above - first) : 0u;
-        const uint32_t full = E / kSplitN, rest = E - full * kSplitN;  // whole tiles, then part of one
-        const uint32_t mine = full > slice ? (full - slice + slices - 1) >> pd.esplit : 0u;
-        const uint32_t tailn = mine * kSplitN + ((full & (slices - 1)) == slice ? rest : 0u);
-        count += tailn * cpe;
-      }
-      if (stop) break;
-      if (i + 1 < nst) stem_next<P, R, W, DB>(x, mult, B, l, ncl);
+      tmem_wait_store();
     }
+    uint32_t n = 0;  // candidates in the warp's queue
+    // exact weights of `cnt` candidates from `at`: a lane takes one and fetches the owner's stem
+    auto check = [&](uint32_t at, uint32_t cnt) {
+      __syncwarp();
+      const bool have = (uint32_t)lane < cnt;
+      const uint32_t item_ = have ? wq.item[at + lane] : 0u;
+      const int src = (int)(item_ & 31u);
+      uint32_t so[RW];
+#pragma unroll
+      for (int q = 0; q < RW; ++q) so[q] = __shfl_sync(FULL, x.s[q], src);
+      const int qo = __shfl_sync(FULL, x.pf.m, src);
+      const uint32_t tl = tails[item_ >> 5];
+      const Tail a = tail_unpack(tl);
+      int wp = 1 << 20, wm = 1 << 20;
+      if (have && a.z > qo) split_weights<P, R, W>(so, a, mult, wp, wm);
+      const bool hit = wp < thr || (l > 0 && wm < thr);
+      if (__any_sync(FULL, hit)) {
+        fpenum::Prefix po;
+        po.m = qo;
+        po.qi = 0;
+        po.Q = __shfl_sync(FULL, (unsigned long long)x.pf.Q, src);
+        po.d = __shfl_sync(FULL, (unsigned long long)x.pf.d, src);
+        note(hit ? hit_key<DB>(B, pair, k, P, g, pass, wp, wm, thr, po, l, tl) : kNoKey);
+      }
+      __syncwarp();
+    };
+    // candidates of the lane's 96 results, those of sign 0, onto the queue:
+    // a word of 32 bits per 32 results (low half: even columns), then one
+    // candidate per lane and round
+    auto scan = [&](const uint32_t (&v0)[16], const uint32_t (&v1)[16], const uint32_t (&v2)[16], uint32_t col0) {
+      uint32_t m0 = 0, m1 = 0, m2 = 0;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        m0 = (m0 >> 1) | (~v0[q] & 0x80008000u);
+        m1 = (m1 >> 1) | (~v1[q] & 0x80008000u);
+        m2 = (m2 >> 1) | (~v2[q] & 0x80008000u);
+      }
+      unsigned any = __ballot_sync(FULL, (m0 | m1 | m2) != 0);
+      do {
+        if (m0 | m1 | m2) {
+          const uint32_t m = m0 ? m0 : m1 ? m1 : m2, col = m0 ? 0u : m1 ? 32u : 64u;
+          const int bit = fpenum::ctz32(m);
+          const uint32_t less = m & (m - 1);
+          if (m0) m0 = less;
+          else if (m1) m1 = less;
+          else m2 = less;
+          wq.item[n + __popc(any & ((1u << lane) - 1u))] =
+              (col0 + col + 2u * (uint32_t)(bit & 15) + (uint32_t)(bit >> 4)) << 5 | (uint32_t)lane;
+        }
+        n += __popc(any);
+        any = __ballot_sync(FULL, (m0 | m1 | m2) != 0);
+        if (n >= 32) {
+          n -= 32;
+          check(n, 32);
+        }
+      } while (any);
+    };
+    int stop = 0;
+    for (uint32_t c = slice; c < tiles && !stop; c += slices) {
+      tc_before_sync();
+      if ((warp & 3) == 0) {
+        if (lane == 0) *(volatile int32_t *)&sh.stop[grp][parity] = finished();
+        group_sync(1 + grp);
+        tc_after_sync();
+        if (elect_one()) {
+          const uint64_t d0 = tile_desc(table + c * (uint32_t)(kSplitN * K), (uint32_t)K);
+          mma_step<false>(tD, tA, d0, kSplitIdesc);
+          if (K > 32) mma_step<true>(tD, tA + 8, d0 + 16, kSplitIdesc);
+          if (K > 64) mma_step<true>(tD, tA + 16, d0 + 32, kSplitIdesc);
+          if (K > 96) mma_step<true>(tD, tA + 24, d0 + 48, kSplitIdesc);
+          mma_commit(mbar);
+        }
+        __syncwarp();
+      } else {
+        group_arrive(1 + grp);
+      }
+      if (!dead && !mbar_wait(mbar, parity)) {
+        dead = true;  // never seen: reported as a timeout, and the rest of the launch drains without results
+        atomicExch(&cd->err, 1);
+      }
+      __syncwarp();
+      stop = *(volatile int32_t *)&sh.stop[grp][parity];
+      parity ^= 1u;
+      tc_after_sync();
+      uint32_t v0[16], v1[16], v2[16];
+      tmem_load16(tD + my_lanes, v0);
+      tmem_load16(tD + my_lanes + 32, v1);
+      tmem_load16(tD + my_lanes + 64, v2);
+      tmem_wait_load(v0, v1, v2);
+      uint32_t a0 = ~0u, a1 = ~0u, a2 = ~0u;
+#pragma unroll
+      for (int q = 0; q < 16; q += 2) {
+        a0 = and3(a0, v0[q], v0[q + 1]);
+        a1 = and3(a1, v1[q], v1[q + 1]);
+        a2 = and3(a2, v2[q], v2[q + 1]);
+      }
+      if (__any_sync(FULL, (~and3(a0, a1, a2) & 0x80008000u) != 0)) scan(v0, v1, v2, c * kSplitN);
+    }
+    if (n) check(0, n);
+    if (act) {
+      // this lane's tails, in the slice's tiles
+      const uint32_t above = tails_above(B, k, t, b, x.pf.m);
+      const uint32_t E = above > first ? min(nb, above - first) : 0u;
+      const uint32_t full = E / kSplitN, rest = E - full * kSplitN;  // whole tiles, then part of one
+      const uint32_t mine = full > slice ? (full - slice + slices - 1) >> pd.esplit : 0u;
+      const uint32_t tailn = mine * kSplitN + ((full & (slices - 1)) == slice ? rest : 0u);
+      count += tailn * cpe;
+    }
+    if (stop) {
+      if (i + 1 < steps) nearly();
+      break;
+    }
+    if (i + 1 < nst) stem_next<P, R, W, DB>(x, mult, B, l, ncl);
   }
 }
 
-// The kernel: bz_kernel's loop (claims, counts, termination tests: the same
-// protocol and the same state) with 512 threads, tail blocks and tensor
-// memory.  One code per launch.
+// Waits bounded by time (globaltimer looked at now and then).
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+               : "=r"(ok)
+               : "r"(bar), "r"(parity)
+               : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool mbar_wait_ns(uint32_t bar, uint32_t parity, unsigned long long limit) {
+  if (mbar_test(bar, parity)) return true;
+  const unsigned long long t0 = globaltimer();
+  for (;;) {
+    for (int i = 0; i < 256; ++i)
+      if (mbar_test(bar, parity)) return true;
+    if (globaltimer() - t0 > limit) return false;
+  }
+}
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 5, 512;" ::: "memory"); }
+
+// The kernel: claims, counts and termination tests follow bz_kernel's
+// protocol on the same state.  One code per launch.  Sixteen warps work;
+// the seventeenth claims: it hands out the next task when the running one
+// nears its end and counts the finished one off while the next runs (in
+// bz_kernel, where thread 0 does both between tasks, a hand-off holds the
+// CTA for about 4 us, a tenth to a third of these searches).  Claiming only
+// near the end keeps the tasks of a pass's end with the CTAs that are free.
 template <int P, int R, int W>
-__global__ void __launch_bounds__(kSplitThreads, 1) split_kernel(const SlotDesc *__restrict__ slots, SlotState *states,
-                                                                 const CtlStatic *__restrict__ ctl, CtlDyn *cdyn,
-                                                                 KParams kp) {
+__global__ void __launch_bounds__(kSplitThreads + 32, 1)
+    split_kernel(const SlotDesc *__restrict__ slots, SlotState *states, const CtlStatic *__restrict__ ctl, CtlDyn *cdyn,
+                 KParams kp) {
   extern __shared__ uint4 smem_raw[];
   char *smem = reinterpret_cast<char *>(smem_raw);
   uint64_t *bcols = reinterpret_cast<uint64_t *>(smem_raw);
-  uint4 *mult4 = smem_raw + kBinomBytes / 16;
-  uint32_t *mult = reinterpret_cast<uint32_t *>(mult4);
-  __shared__ Claim s_cl;
   __shared__ ClaimCache s_cc;
   __shared__ SegCache<kSplitSegCache, SplitSeg> s_sc;
   __shared__ __align__(16) PassDesc s_pc[kSplitPassCache];
   __shared__ SplitShared s_sh;
-  __shared__ __align__(8) unsigned long long s_mbar[kSplitGroups];
   __shared__ uint32_t s_tmem;
-  __shared__ int s_npc, s_cmd, s_stage, s_build, s_over;
-  __shared__ unsigned long long s_count;
-  __shared__ int s_staged_j, s_built_t, s_built_block, s_built_n;
 
   const CtlStatic cs = *ctl;
-  const int tid = threadIdx.x;
-  int rr = 0;
-  unsigned long long wait_t0 = 0;
+  const int tid = threadIdx.x, threads = kSplitThreads + 32;
   const unsigned long long t_start = globaltimer();
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  // longest wait for another warp: past every bounded wait of the claims
+  const unsigned long long wait_ns = 2 * kp.wait_limit_ns + 60000000000ull;
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int i = 0; i < kSplitGroups; ++i)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s_mbar[i])) : "memory");
+    for (int i = 0; i < kSplitGroups; ++i) mbar_init(smem_u32(&s_sh.product[i]), 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&s_sh.full[i]), 1);
+      mbar_init(smem_u32(&s_sh.near[i]), kSplitGroups);
+      mbar_init(smem_u32(&s_sh.done[i]), kSplitWarps);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    s_staged_j = -1;
-    s_built_t = -1;
-    s_built_block = -1;
-    s_built_n = 0;
-    s_cc.slot = -1;
+    s_sh.best_key = 0;
+    s_sh.finished = 0;
+    s_cc.sd = load_nc(&slots[0]);  // one thread per CTA, through L1: every CTA reads the same bytes at once
+    s_cc.slot = 0;
+    s_cc.gen = s_cc.sd.seq & kGenMask;
     s_cc.P = -1;
-    s_cc.gen = 0;
     s_cc.sleep_ns = 128;
     s_cc.busy_note = 0;
     s_sc.slot = -1;
     s_sc.pass = -1;
     s_sc.gen = 0;
-    s_npc = 0;
-    s_over = 0;
-    s_cc.sd = load_nc(&slots[0]);  // one thread per CTA, through L1: every CTA reads the same bytes at once
   }
   {
     const uint4 *bsrc = reinterpret_cast<const uint4 *>(cs.binom->cols);
-    for (int i = tid; i < kBinomBytes / 16; i += kSplitThreads) smem_raw[i] = __ldg(bsrc + i);
+    for (int i = tid; i < kBinomBytes / 16; i += threads) smem_raw[i] = __ldg(bsrc + i);
   }
   const fpenum::BinomCols binom{bcols};
   tc_before_sync();
@@ -628,12 +666,11 @@ __global__ void __launch_bounds__(kSplitThreads, 1) split_kernel(const SlotDesc 
   {
     // pass descriptors and segments: nothing in the launch writes them
     const uint4 *src = reinterpret_cast<const uint4 *>(s_cc.sd.passes);
-    for (int i = tid; i < npc * (int)(sizeof(PassDesc) / 16); i += kSplitThreads)
-      reinterpret_cast<uint4 *>(s_pc)[i] = __ldg(src + i);
+    for (int i = tid; i < npc * (int)(sizeof(PassDesc) / 16); i += threads) reinterpret_cast<uint4 *>(s_pc)[i] = __ldg(src + i);
     const int nsegs = s_cc.sd.nsegs;
     if (nsegs > 0 && nsegs <= kSplitSegCache) {
       const uint4 *ssrc = reinterpret_cast<const uint4 *>(s_cc.sd.passes + np);
-      for (int i = tid; i < nsegs; i += kSplitThreads) reinterpret_cast<uint4 *>(s_sc.seg)[i] = __ldg(ssrc + i);
+      for (int i = tid; i < nsegs; i += threads) reinterpret_cast<uint4 *>(s_sc.seg)[i] = __ldg(ssrc + i);
       if (tid == 0) {
         s_sc.slot = 0;
         s_sc.gen = s_cc.sd.seq & kGenMask;
@@ -642,89 +679,134 @@ __global__ void __launch_bounds__(kSplitThreads, 1) split_kernel(const SlotDesc 
     }
   }
   __syncthreads();
-  const SlotDesc &sd = s_cc.sd;
-  const int K = sd.split_k;
-  uint32_t *tails = reinterpret_cast<uint32_t *>(smem + split_off_tails(sd.k, P, sd.rwpad));
-  char *table = smem + split_off_table(sd.k, P, sd.rwpad, sd.split_cap);
-  const int grp = warp / (kSplitGroup / 32);
-  const uint32_t mbar = smem_u32(&s_mbar[grp]);
-  uint32_t parity = 0;
-  if (tid == 0) {
-    s_cc.slot = 0;
-    s_cc.gen = s_cc.sd.seq & kGenMask;
-    s_npc = npc;
-    if (np > 0) {
-      s_cc.pd = s_pc[0];
-      s_cc.P = 0;
-    }
-  }
-  __syncthreads();
-  for (;;) {
-    if (tid == 0) {
-      const int cmd =
-          s_over ? kCmdExit : claim(slots, states, cs, kp, cdyn, rr, wait_t0, t_start, &s_cl, s_cc, s_sc, s_pc, s_npc, binom);
-      s_cmd = cmd;
-      if (cmd == kCmdRun) {
-        s_stage = !s_cl.skip && s_cc.pd.j != s_staged_j;
-        if (s_stage) {
-          s_staged_j = s_cc.pd.j;
-          s_built_t = -1;
-        }
-        s_build = 0;
-        if (!s_cl.skip && s_cc.pd.g >= 2) {
-          // a direct pass needs the packed tails only, which a built table of the same block has too
-          const int need = s_cc.pd.direct ? 1 : 2, bt = s_cc.pd.tail_rows << 16 | (int)s_cc.pd.block;
-          if (s_built_t != bt || s_built_block != (int)s_cl.block || s_built_n < need) {
-            s_build = need;
-            s_built_t = bt;
-            s_built_block = (int)s_cl.block;
-            s_built_n = need;
+  if (warp == kSplitWarps) {
+    if ((tid & 31) == 0) {
+      // what the tables hold: the set, the block (tail length and size, index) and how much of it
+      int rr = 0, staged_j = -1, built = -1, built_n = 0;
+      unsigned int built_block = 0;
+      unsigned long long wait_t0 = 0;
+      if (np > 0) {
+        s_cc.pd = s_pc[0];
+        s_cc.P = 0;
+      }
+      uint32_t head = 0, tail = 0;  // tasks handed out, tasks counted off
+      unsigned long long since = 0;  // when the scheduler began to wait for a running task
+      bool over = false;
+      for (;;) {
+        if (!over && head - tail < 2) {
+          // one task runs: the next is claimed once its warpgroups are in their last steps
+          const uint32_t r = (head - 1) & 1u, rp = ((head - 1) >> 1) & 1u;
+          if (head == tail || mbar_test(smem_u32(&s_sh.near[r]), rp) || mbar_test(smem_u32(&s_sh.done[r]), rp)) {
+            SplitTask &tk = s_sh.task[head & 1u];
+            if (head != tail) s_cc.sleep_ns = 128;  // a finished task must not wait for the back-off
+            const int cmd = claim(slots, states, cs, kp, cdyn, rr, wait_t0, t_start, &tk.cl, s_cc, s_sc, s_pc, npc, binom);
+            if (cmd == kCmdExit) {
+              over = true;
+            } else if (cmd == kCmdRun) {
+              tk.pd = s_cc.pd;
+              tk.cmd = kCmdRun;
+              tk.count = 0;
+              tk.stage = tk.build = tk.drop = 0;
+              if (!tk.cl.skip) {
+                // a direct pass needs the packed tails only, which a built table of the same block has too
+                const int need = tk.pd.g < 2 ? 0 : tk.pd.direct ? 1 : 2, bt = tk.pd.tail_rows << 16 | (int)tk.pd.block;
+                tk.stage = staged_j != tk.pd.j;
+                if (need && (tk.stage || built != bt || built_block != tk.cl.block || built_n < need)) {
+                  tk.build = need;
+                  built = bt;
+                  built_block = tk.cl.block;
+                  built_n = need;
+                } else if (tk.stage) {
+                  built = -1;
+                }
+                staged_j = tk.pd.j;
+              }
+              mbar_arrive(smem_u32(&s_sh.full[head & 1u]));
+              ++head;
+              continue;
+            }
           }
         }
-        s_sh.next = 0;
+        if (head == tail) {
+          if (over) break;
+          continue;
+        }
+        const uint32_t o = tail & 1u, op = (tail >> 1) & 1u;
+        {  // pass on the best key and the finished flag (the loads pace this loop)
+          const unsigned long long key = ld_vol(&states[0].best_key);
+          const int fin = ld_vol(&states[0].finished);
+          *(volatile unsigned long long *)&s_sh.best_key = key;
+          *(volatile int32_t *)&s_sh.finished = fin;
+        }
+        if (mbar_test(smem_u32(&s_sh.done[o]), op)) {
+          const SplitTask &tk = s_sh.task[o];
+          if (tk.count) {
+            atomicAdd(&states[0].enumerated, tk.count);
+            atomicAdd(&cs.aux->pass_count[tk.cl.pass], tk.count);
+          }
+          if (finish_task(cs, kp, cdyn, s_cc.sd, &states[0], cs.aux, 0, tk.cl.pass, tk.pd, tk.cl.ndone, s_pc, npc))
+            over = true;
+          ++tail;
+          since = 0;
+        } else if (since == 0) {
+          since = globaltimer();
+        } else if (globaltimer() - since > wait_ns) {
+          atomicExch(&cdyn->err, 1);  // a warp never finished: report a timeout
+          break;
+        }
       }
-      s_count = 0;
+      s_sh.task[head & 1u].cmd = kCmdExit;
+      mbar_arrive(smem_u32(&s_sh.full[head & 1u]));
     }
-    __syncthreads();
-    const int cmd = s_cmd;
-    if (cmd == kCmdExit) break;
-    if (cmd == kCmdWait) {
-      __syncthreads();
-      continue;
-    }
-    if (s_stage) {
-      const int nv = split_mult_words(sd.k, P, sd.rwpad) / 4;
-      const uint4 *src = reinterpret_cast<const uint4 *>(sd.table + (size_t)s_cc.pd.j * (size_t)table_words(sd));
-      for (int i = tid; i < nv; i += kSplitThreads) mult4[i] = __ldg(src + i);
-      __syncthreads();
-    }
-    if (s_build) {
-      const uint32_t etot = tails_above(binom, sd.k, s_cc.pd.tail_rows, P - 1, -1), first = s_cl.block * s_cc.pd.block;
-      build_tails<P, R, W>(tails, table, mult, binom, sd.k, s_cc.pd.tail_rows, first, min(s_cc.pd.block, etot - first), K,
-                           sd.split_nu, s_build == 2);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the tensor cores read the table
-      __syncthreads();
-    }
-    unsigned long long count = 0;
-    SlotAux *ax = cs.aux;
-    if (!s_cl.skip) {
-      if (s_cc.pd.g == 1) {
-        if (s_cl.ulo == 0) task_rows<P, R, W>(sd, s_cl.pass, mult, s_cl.U, &states[0], ax, count);
+    __syncwarp();
+  } else {
+    const SlotDesc &sd = s_cc.sd;
+    const int K = sd.split_k;
+    uint32_t *mult = reinterpret_cast<uint32_t *>(smem + kBinomBytes);
+    uint32_t *tails = reinterpret_cast<uint32_t *>(smem + split_off_tails(sd.k, P, sd.rwpad));
+    char *table = smem + split_off_table(sd.k, P, sd.rwpad, sd.split_cap);
+    const int grp = warp / (kSplitGroup / 32);
+    uint32_t parity = 0;
+    for (uint32_t n = 0;; ++n) {
+      SplitTask &tk = s_sh.task[n & 1u];
+      if (!mbar_wait_ns(smem_u32(&s_sh.full[n & 1u]), (n >> 1) & 1u, wait_ns)) {
+        atomicExch(&cdyn->err, 1);
+        break;
+      }
+      __syncwarp();
+      if (tk.cmd == kCmdExit) break;
+      if (tk.stage || tk.build) {
+        if (tid == 0) tk.drop = *(volatile int32_t *)&s_sh.finished;
+        workers_sync();  // every warp has left the previous task: its tables may go
+        if (tk.stage && !tk.drop) {
+          const int nv = split_mult_words(sd.k, P, sd.rwpad) / 4;
+          const uint4 *src = reinterpret_cast<const uint4 *>(sd.table + (size_t)tk.pd.j * (size_t)table_words(sd));
+          for (int i = tid; i < nv; i += kSplitThreads) reinterpret_cast<uint4 *>(mult)[i] = __ldg(src + i);
+          workers_sync();
+        }
+        if (tk.build && !tk.drop) {
+          const uint32_t etot = tails_above(binom, sd.k, tk.pd.tail_rows, P - 1, -1), first = tk.cl.block * tk.pd.block;
+          build_tails<P, R, W>(tails, table, mult, binom, sd.k, tk.pd.tail_rows, first, min(tk.pd.block, etot - first), K,
+                               sd.split_nu, tk.build == 2);
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the tensor cores read the table
+          workers_sync();
+        }
+      }
+      unsigned long long count = 0;
+      const uint32_t near = smem_u32(&s_sh.near[n & 1u]);
+      if (tk.cl.skip || tk.drop || tk.pd.g == 1) {
+        if ((tid & (kSplitGroup - 1)) == 0) mbar_arrive(near);
+        if (!tk.cl.skip && !tk.drop && tk.cl.ulo == 0) task_rows<P, R, W>(sd, tk.cl.pass, mult, tk.cl.U, &states[0], cs.aux, count);
       } else {
-        task_split<P, R, W>(sd, s_cc.pd, s_cl, mult, tails, smem_u32(table), tmem, mbar, parity, binom, s_sh, &states[0],
-                            ax, cdyn, count);
+        task_split<P, R, W>(sd, tk.pd, tk.cl, mult, tails, smem_u32(table), tmem, smem_u32(&s_sh.product[grp]), parity, near,
+                            binom, s_sh, &states[0], cs.aux, cdyn, count);
       }
-    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
-    if ((tid & 31) == 0 && count) atomicAdd(&s_count, count);
-    __syncthreads();
-    if (tid == 0) {
-      if (s_count) {
-        atomicAdd(&states[0].enumerated, s_count);
-        atomicAdd(&ax->pass_count[s_cl.pass], s_count);
+      for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
+      if ((tid & 31) == 0) {
+        if (count) atomicAdd(&tk.count, count);
+        mbar_arrive(smem_u32(&s_sh.done[n & 1u]));
       }
-      if (finish_task(cs, kp, cdyn, s_cc.sd, &states[0], ax, 0, s_cl.pass, s_cc.pd, s_cl.ndone, s_pc, s_npc)) s_over = 1;
     }
   }
   tc_before_sync();

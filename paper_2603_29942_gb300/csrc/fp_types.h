@@ -58,13 +58,12 @@ struct PassDesc {
   uint32_t seg_off;        // pair-leaf passes: first segment of the pass in the code's segment list
   uint32_t nseg;           // pair-leaf passes: its segments (0: a one-row-leaf pass)
   uint32_t task_off;       // a slice of the pass (fpcode_prepared_pass_slice): its first task in the pass's plan
-  // Split passes (fp_split.cuh; then seg_off and nseg count SplitSegs, and
-  // `unit` is the stems per lane and item).
+  // Split passes (fp_split.cuh; then seg_off and nseg count SplitSegs).
   uint64_t ncl;            // coefficient vectors per stem row subset
   uint32_t block;          // tails per block
   uint8_t tail_rows;       // rows of a tail (2 or 3)
   uint8_t direct;          // 1: few codewords, every weight exact
-  uint8_t esplit;          // log2 of the slices of a block's tails that are items of their own
+  uint8_t esplit;          // log2 of the warpgroups that share a task's stems and split its tails
   uint8_t pad0;
 };
 
