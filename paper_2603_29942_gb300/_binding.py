@@ -856,6 +856,15 @@ def fpcode_test_split_pass(prep: Prepared, pass_index: int, ctas: int = 152, tai
     return None if n < 0 else keys[:min(n, cap)]
 
 
+def fpcode_test_split_runs(prep: Prepared, pass_index: int, ctas: int = 152) -> int:
+    """Runs of tasks in the tensor-core kernel's plan of a pass (g >= 2)."""
+    n = lib().fpcode_test_split_pass(prep.handle, int(pass_index), int(ctas), -1, 1, 1, 0,
+                                     (ctypes.c_uint64 * 1)(), 1)
+    if n < 0:
+        raise FpcodeError(EINVAL, "fpcode_test_split_pass")
+    return int(n)
+
+
 def fpcode_test_key_coefficients(prep: Prepared, key: int):
     """(g, j, coefficients) of the codeword a packed key stands for, or None."""
     g = ctypes.c_int(0)

@@ -783,7 +783,7 @@ TailCut cut_tails(const Prepared &P, int t, uint32_t cap) {
   TailCut c;
   c.t = t;
   const uint32_t nblk = (etot + cap - 1) / cap;
-  if (nblk > 255) return c;  // the run's field
+  if (nblk > 128) return c;  // with the runs of the first block, a pass stays within the kernel's copy of one pass's runs
   c.nb = ((etot + nblk - 1) / nblk + N - 1) / N * N;
   for (uint32_t first = 0; first < etot; first += c.nb) {
     TailCut::Block x;
@@ -1351,6 +1351,7 @@ int64_t fpcode_test_split_pass(fpcode_prepared *prep, int pass, int ctas, int ta
     if (fph::digit_bits_of(P.p) == 1) split_walk<1>(P, d, pass, lo, hi, blk, zhi, emit);
     else split_walk<4>(P, d, pass, lo, hi, blk, zhi, emit);
   };
+  if (tail_rows < 0) return (int64_t)d.nseg;
   if (tail_rows == 0) {  // the plan's own tasks
     for (uint64_t t = 0; t < d.ntasks; ++t) {
       uint64_t lo = 0, hi = 0;

@@ -931,6 +931,7 @@ struct Claim {  // the task taken (its code's and pass's descriptors: the ClaimC
 constexpr int kSegPass = 192;
 constexpr int kSplitSegCache = 320;  // the split kernel's copies of segments and pass descriptors
 constexpr int kSplitPassCache = 24;
+static_assert(kSegPass >= kSplitPassSegs && kSplitSegCache >= kSplitPassSegs, "copies of one pass's segments");
 template <int N, class S = PairSeg>
 struct alignas(16) SegCache {  // segments are copied in pieces of their size, up to 16 bytes
   using Seg = S;

@@ -38,6 +38,10 @@ struct SplitSeg {
 };
 static_assert(sizeof(SplitSeg) == 16, "SplitSeg layout");
 
+// Runs of one pass at most (the kernel's copy of the runs of the pass it
+// claims from, when a code has too many to keep them all).
+constexpr int kSplitPassSegs = 192;
+
 // Units [lo, hi) of task t of a split pass whose runs are seg[0 .. nseg);
 // returns the run.
 FPK_HD SplitSeg split_task(const SplitSeg *seg, int nseg, uint64_t t, uint64_t *lo, uint64_t *hi) {

@@ -61,6 +61,24 @@ def test_split_plan_covers_early_passes(p, n, k, ctas, lib):
         assert len(keys) == size and len(np.unique(keys)) == size
 
 
+@pytest.mark.parametrize("p", [3, 5, 7])
+def test_split_plan_runs_fit_the_kernels_copy(p, lib):
+    """No pass of any shape has more than 192 runs of tasks (the kernel copies
+    those of one pass when a code has too many in all)."""
+    most, seen = 0, 0
+    for k in (5, 12, 20, 28, 36, 40, 43, 50, 57, 64):
+        for red in (6, 20, 33, 41, 70, 120):
+            pr = _prep(inputs.single_code(1, p, k + red, k))
+            if pr is None:
+                continue
+            for ctas in (152, 7):
+                for i, x in enumerate(B.fpcode_prepared_passes(pr)):
+                    if x[0] >= 2 and x[1] == 0:
+                        most = max(most, B.fpcode_test_split_runs(pr, i, ctas))
+                        seen += 1
+    assert seen > 100 and 1 <= most <= 192
+
+
 def test_which_codes_are_split(lib):
     """p = 3, 5, 7 with the leaf form left to the library; not with a leaf
     form asked for, other primes, or rows that hold too many class values."""
