@@ -117,7 +117,7 @@ int fpcode_test_prepare_split(int p, int n, int k, const uint8_t *G, const fpcod
  * order, as packed keys of weight 0 in the code's leaf form: the pass's own
  * tasks planned for `ctas` CTAs (tail_rows = 0), or the whole pass with
  * tails of tail_rows rows in blocks of `block`, tasks of `unit` times 128
- * stems and 1 << esplit (1, 2 or 4) slices; tail_rows < 0
+ * stems, each warpgroup on its own or (esplit) on a slice of the tails; tail_rows < 0
  * returns the runs of tasks of the pass's plan instead.  Returns their number (entries past max not
  * written), or -1 (no such pass, or the code is not searched this way). */
 int64_t fpcode_test_split_pass(fpcode_prepared *prep, int pass, int ctas, int tail_rows, int block, int unit, int esplit,

@@ -290,7 +290,7 @@ int smem_for(const std::vector<const fph::Prepared *> &codes) {
 const void *kernel_of(const fph::Prepared &P) {
   return P.split ? fpk::kernel_split(P.p, P.W) : kernel_for(P.variant);
 }
-int threads_of(const fph::Prepared &P) { return P.split ? fpk::kSplitThreads + 32 : fpk::kThreads; }
+int threads_of(const fph::Prepared &P) { return P.split ? fpk::kSplitLaunch : fpk::kThreads; }
 
 // with_state: the host image also holds the first state (zeroed
 // bookkeeping, the bound in the best key) and one copy takes both, so the
@@ -709,8 +709,7 @@ int fpcode_min_distance_batch(int num, const fpcode_desc *codes, void *stream, c
         fpcode_opts oi = o;
         if (!per_variant) oi.pair_leaves = 0;  // the batched kernels take one-row leaves
         if (codes[i].budget) oi.budget = codes[i].budget;
-        status[i] = fph::prepare(codes[i].p, codes[i].n, codes[i].k, codes[i].G, oi, preps[i].get());
-        preps[i]->split = false;  // many codes share a launch: the leaf kernels
+        status[i] = fph::prepare(codes[i].p, codes[i].n, codes[i].k, codes[i].G, oi, preps[i].get(), fph::SplitUse::kNever);
       }
     };
     std::vector<std::thread> pool;

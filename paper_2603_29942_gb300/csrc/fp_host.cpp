@@ -243,9 +243,10 @@ double expected_work(int p, int n, int k) {
 }
 // Tensor-core kernel (pair_leaves 2): from this much expected work on, and
 // with at least this many redundant symbols (its class comparison needs
-// some).  Measured per call, leaf kernels against it: F_7 [40,20] (4.2e7
-// codewords) 80 against 112 us, F_3 [80,40] (2.7e8) 177 against 161, F_5
-// [51,24] (3.0e8) 429 against 169, F_7 [52,19] (2.9e10) 17 400 against 2 890.
+// some).  Measured, leaf kernels against it: F_7 [40,20] (4.2e7 codewords)
+// kernel 46 against 50 us; whole searches of F_3 [80,40] (2.7e8) 174 against
+// 119 us, F_5 [51,24] (3.0e8) 431 against 126, F_7 [52,19] (2.9e10) 17 390
+// against 1 965.
 constexpr double kSplitWork = 1e8;
 constexpr int kSplitMinRed = 4;
 // Dynamic shared memory of one of its CTAs: 227 KiB less the kernel's own.
@@ -254,7 +255,7 @@ constexpr double kPairWork = 1e8;  // pair_leaves 2: pair leaves from this much 
 
 }  // namespace
 
-int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prepared *P, bool any_size) {
+int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prepared *P, SplitUse use) {
   auto t0 = std::chrono::steady_clock::now();
   if (!is_odd_prime(p)) {
     set_error("p must be an odd prime below 256");
@@ -494,8 +495,9 @@ int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prep
   // by its budget.
   P->split = false;
   P->split_k = P->split_nu = P->split_cap = 0;
-  if (opts.pair_leaves == 2 && (p == 3 || p == 5 || p == 7) && k >= 3 && n - k >= kSplitMinRed &&
-      (any_size || std::min((double)total, expected_work(p, n, k)) >= kSplitWork)) {
+  if (use != SplitUse::kNever && opts.pair_leaves == 2 && (p == 3 || p == 5 || p == 7) && k >= 3 &&
+      n - k >= kSplitMinRed &&
+      (use == SplitUse::kAny || ((double)total >= kSplitWork && expected_work(p, n, k) >= kSplitWork))) {
     const int K = fpk::split_k(p, n - k, &P->split_nu);
     if (K > 0) {
       const int room = kSplitSmemMax - fpk::split_off_tails(k, p, P->rwpad) - 256;
@@ -751,7 +753,7 @@ int split_smem_bytes(const Prepared &P) {
 
 namespace {
 
-// Clocks of an SM (its four warpgroups at work) for the parts of a split
+// Clocks of an SM (its warpgroups at work) for the parts of a split
 // pass, from traced searches: a stem step of 128 lanes, one tile of results
 // (the tensor pipe's time, or the warps' for short rows), the build of a
 // block of n tails, the start of a task's lanes.
@@ -759,7 +761,10 @@ constexpr double kStepClocks = 500, kStartClocks = 1500;
 inline double tile_clocks(int K) { return std::max(150.0, 1.5 * K); }
 inline double build_clocks(double n) { return 2500 + 2.2 * n; }
 constexpr double kTaskClocks = 6000;         // least work of a task
-constexpr uint64_t kDirectCombos = 1 << 19;  // stem-tail pairs of a pass up to which every weight is computed exactly
+// Stem-tail pairs of a pass up to which every weight is computed exactly,
+// which spreads an early pass wide before any record lowers the threshold
+// (F_3 [80,40]: 87 us with 2^19, 91 with 2^17, 96 with 2^13).
+constexpr uint64_t kDirectPairs = 1 << 19;
 
 // One way to cut a code's tails: t rows, blocks of nb.  It depends on the
 // code's shape only, so it is worked out once for all passes.
@@ -858,7 +863,7 @@ void plan_split(Prepared *P, int ctas) {
     double total = 0;
     const TailCut *cut = nullptr;
     const uint64_t combos = g == 2 ? d.size : d.size / 2;
-    if (combos <= kDirectCombos) {
+    if (combos <= kDirectPairs) {
       d.direct = 1;
       nb = fpk::tails_above(binom(), k, 2, b, -1);
     } else {
@@ -886,7 +891,7 @@ void plan_split(Prepared *P, int ctas) {
     auto add = [&](uint32_t item0, uint32_t item1, uint64_t per, uint32_t block, int zhi) {
       if (item0 >= item1) return;
       fpk::SplitSeg s{};
-      per = std::min<uint64_t>(std::max<uint64_t>(per, 1), 65532);
+      per = std::min<uint64_t>(std::max<uint64_t>(per, 1), 65535 / fpk::kSplitGroups * fpk::kSplitGroups);
       tasks += (uint32_t)((item1 - item0 + per - 1) / per);
       s.task_end = tasks;
       s.item0 = item0;
@@ -899,7 +904,7 @@ void plan_split(Prepared *P, int ctas) {
     if (d.direct) {
       // runs of stems with about the same number of tails, as many to a task
       // as give every warpgroup of the grid the same work
-      d.esplit = g == 2 ? 2 : 0;
+      d.esplit = g == 2 ? 1 : 0;
       auto stem_clocks = [&](int q) {
         return 400.0 + 800.0 * (double)((fpk::tails_above(binom(), k, t, b, q) + fpk::kSplitGroup - 1) / fpk::kSplitGroup);
       };
@@ -907,24 +912,23 @@ void plan_split(Prepared *P, int ctas) {
       for (int q = std::max(l - 1, 0); l > 0 && q < k - 2; ++q) work += (double)(binom().c[q][l - 1] * d.ncl) * stem_clocks(q);
       const uint32_t items = (uint32_t)(l > 0 ? binom().c[k - 2][l] * d.ncl : 1);
       // the passes of one level run side by side, one per information set
-      const double target = std::max(3000.0, work * std::min(P->m, 4) / (4 * C));
+      const double target = std::max(3000.0, work * std::min(P->m, 4) / (fpk::kSplitGroups * C));
       uint32_t at = 0;
       for (int q = std::max(l - 1, 0); at < items;) {
         const double c = stem_clocks(l > 0 ? q : -1);
         int q1 = q + 1;
         while (l > 0 && q1 < k - 2 && stem_clocks(q1) * 1.3 >= c) ++q1;
         const uint32_t end = l > 0 && q1 < k - 2 ? (uint32_t)(binom().c[q1][l] * d.ncl) : items;
-        add(at, end, l > 0 ? 4 * std::max<uint64_t>(1, (uint64_t)(target / c)) : 1, 0, k - 2);
+        add(at, end, l > 0 ? fpk::kSplitGroups * std::max<uint64_t>(1, (uint64_t)(target / c)) : 1, 0, k - 2);
         at = std::max(at, end);
         q = q1;
       }
     } else {
-      // a task of least size: 4 units with all warpgroups on their own, or
-      // 2 or 1 with their tails split
+      // a task of least size: one unit for each warpgroup, or one in all with its tails split
       const double unit_max = kStepClocks + tile * cut->blocks[0].tiles;
       const double target0 = std::max(kTaskClocks, std::min(total / C, 4 * kTaskClocks));
-      d.esplit = 4 * unit_max <= 1.5 * target0 ? 0 : 2 * unit_max <= 1.5 * target0 ? 1 : 2;
-      const uint64_t parts = 4u >> d.esplit;
+      d.esplit = fpk::kSplitGroups * unit_max <= 1.5 * target0 ? 0 : 1;
+      const uint64_t parts = d.esplit ? 1 : fpk::kSplitGroups;
       double rem = total;
       for (uint32_t blk = 0; blk < cut->blocks.size(); ++blk) {
         const TailCut::Block &x = cut->blocks[blk];
@@ -1285,24 +1289,21 @@ void split_walk(const fph::Prepared &P, const fpk::PassDesc &d, int pass, uint64
   const fpenum::Binom &B = fph::binom();
   const int k = P.k, b = P.p - 1, g = d.g, t = d.tail_rows, l = g - t;
   const uint32_t etot = fpk::tails_above(B, k, t, b, -1), first = block * d.block;
-  const uint32_t nb = std::min(d.block, etot - first), slices = 1u << d.esplit, parts = 4u >> d.esplit;
+  const uint32_t nb = std::min(d.block, etot - first);
+  const uint32_t slices = d.esplit ? fpk::kSplitGroups : 1, parts = d.esplit ? 1 : fpk::kSplitGroups;
   const uint64_t ns = l > 0 ? B(zhi, l) * d.ncl : 1;
   const uint32_t lanes = d.direct ? 1 : fpk::kSplitGroup, tile = d.direct ? fpk::kSplitGroup : fpk::kSplitN;
   const uint64_t share = (hi - lo + parts - 1) / parts;
-  for (uint32_t grp = 0; grp < 4; ++grp) {
-    const uint32_t part = grp >> d.esplit, slice = grp & (slices - 1);
+  for (uint32_t grp = 0; grp < fpk::kSplitGroups; ++grp) {
+    const uint32_t part = d.esplit ? 0 : grp, slice = d.esplit ? grp : 0;
     const uint64_t u0 = std::min(lo + part * share, hi), steps = std::min(u0 + share, hi) - u0, J0 = u0 * lanes;
     if (steps == 0 || J0 >= ns) continue;
     const int q0 = l > 0 ? fpk::comb_floor(B, l - 1, k - t - 1, l, d.ncl, J0) : -1;
     const uint32_t tiles = (std::min(nb, fpk::tails_above(B, k, t, b, q0) - first) + tile - 1) / tile;
     for (uint32_t lane = 0; lane < lanes; ++lane) {
       const uint64_t J = J0 + lane * steps, nst = J < ns ? std::min(steps, ns - J) : 0;
-      fpenum::Prefix pf{-1, 0, 0, 0};
-      uint64_t ci = 0, nq = 1;
-      if (nst && l > 0) {
-        pf = fpk::stem_unrank<DB>(B, J, k, t, l, b, d.ncl, &ci);
-        nq = B(pf.m, l - 1);
-      }
+      fpk::StemPos pf{-1, 0, 0};
+      if (nst && l > 0) pf = fpk::stem_unrank<DB>(B, J, k, t, l, b, d.ncl);
       for (uint64_t i = 0; i < nst; ++i) {
         for (uint32_t c = slice; c < tiles; c += slices)
           for (uint32_t e = c * tile; e < std::min((c + 1) * tile, nb); ++e) {
@@ -1312,7 +1313,7 @@ void split_walk(const fph::Prepared &P, const fpk::PassDesc &d, int pass, uint64
               emit(fpk::split_key<DB>(B, P.pair, k, P.p, g, (uint32_t)pass, 0, pf, l, a, sign));
           }
         int dir = 1;
-        if (l > 0 && i + 1 < nst) fpk::stem_advance<DB>(B, pf, ci, nq, d.ncl, b, l, &dir);
+        if (l > 0 && i + 1 < nst) fpk::stem_advance<DB>(pf, b, l, &dir);
       }
     }
   }
@@ -1325,7 +1326,7 @@ int fpcode_test_prepare_split(int p, int n, int k, const uint8_t *G, const fpcod
   *out = nullptr;
   fpcode_prepared *prep = new (std::nothrow) fpcode_prepared();
   if (!prep) return FPCODE_ENOMEM;
-  const int s = fph::prepare(p, n, k, G, *opts, &prep->host, true);
+  const int s = fph::prepare(p, n, k, G, *opts, &prep->host, fph::SplitUse::kAny);
   if (s || !prep->host.split) {
     delete prep;
     return s ? s : FPCODE_EINVAL;
@@ -1361,7 +1362,7 @@ int64_t fpcode_test_split_pass(fpcode_prepared *prep, int pass, int ctas, int ta
     return n;
   }
   const int l = d.g - tail_rows;
-  if (tail_rows < 2 || tail_rows > 3 || l < 0 || block < 1 || unit < 1 || esplit < 0 || esplit > 2) return -1;
+  if (tail_rows < 2 || tail_rows > 3 || l < 0 || block < 1 || unit < 1 || esplit < 0 || esplit > 1) return -1;
   d.direct = 0;
   d.tail_rows = (uint8_t)tail_rows;
   d.block = (uint32_t)block;

@@ -83,8 +83,12 @@ int task_share_of(const fpcode_opts &o, bool last);
 
 // Elimination, information sets, multiples, schedule.  Returns an fpcode
 // status; the error text is set on failure.
-// any_size: the tensor-core kernel also for a search too small for it (tests).
-int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prepared *out, bool any_size = false);
+// Whether the tensor-core kernel may take the code: with the leaf form left
+// to the library (pair_leaves 2) and enough work; any amount (tests); never
+// (a code that shares its launch with others).
+enum class SplitUse { kAlone, kAny, kNever };
+int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prepared *out,
+            SplitUse use = SplitUse::kAlone);
 
 // Tasks and prefixes per lane of every pass for a grid of `ctas` CTAs.
 // fixed_pl > 0: tasks of fixed_pl prefixes per lane everywhere.  Else a pass

@@ -80,9 +80,8 @@ extern "C" int fpcode_min_distance_noalloc(int p, int n, int k, const uint8_t *G
   fpcode_opts o;
   fpcode_opts_default(&o);
   fph::Prepared P;
-  int s = fph::prepare(p, n, k, G, o, &P);
+  int s = fph::prepare(p, n, k, G, o, &P, fph::SplitUse::kNever);  // the fixed array holds the leaf kernels' plan
   if (s) return s;
-  P.split = false;  // the fixed array holds the leaf kernels' plan
 
   // layout inside the array: [binom][CtlStatic][SlotDesc][passes, segments][table][state][dyn][aux][flags].
   // The pair-leaf plan (made below, for the grid) has at most one segment

@@ -271,7 +271,7 @@ int fpcode_serve_submit(fpcode_server *s, const fpcode_desc *code, uint64_t *tic
   o.pair_leaves = 0;  // the serving kernels take one-row leaves
   if (code->budget) o.budget = code->budget;
   std::unique_ptr<fph::Prepared> P(new fph::Prepared());
-  int st = fph::prepare(code->p, code->n, code->k, code->G, o, P.get());
+  int st = fph::prepare(code->p, code->n, code->k, code->G, o, P.get(), fph::SplitUse::kNever);
   if (st) return st;
   if (P->variant >= 12) {
     fph::set_error("serve: p must be 3, 5 or 7");

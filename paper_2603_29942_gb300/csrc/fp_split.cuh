@@ -27,8 +27,8 @@ namespace fpk {
 // One run of tasks of a split pass: units [item0, item1) of one tail block,
 // `per` to a task.  A unit is 128 stems (tensor-core passes) or one stem
 // (direct passes).  The four warpgroups of a CTA share a task's units
-// evenly, or (esplit 1, 2) half or all of them share the same units and
-// take interleaved slices of the block's tails.
+// evenly, or (esplit) all take the same units and interleaved slices of the
+// block's tails.
 struct SplitSeg {
   uint32_t task_end;  // tasks of the pass up to the end of this run
   uint32_t item0, item1;
@@ -59,8 +59,10 @@ FPK_HD SplitSeg split_task(const SplitSeg *seg, int nseg, uint64_t t, uint64_t *
   return g;
 }
 
-constexpr int kSplitThreads = 512;  // working threads per CTA of the tensor-core kernel (one more warp claims)
-constexpr int kSplitGroup = 128;    // lanes per warpgroup: rows of one accumulator tile
+constexpr int kSplitGroups = 4;     // warpgroups that work in a CTA (one more warp claims)
+constexpr int kSplitGroup = 128;    // their lanes: rows of one accumulator tile
+constexpr int kSplitThreads = kSplitGroups * kSplitGroup;
+constexpr int kSplitLaunch = kSplitThreads + 128;  // with the claiming warp's warpgroup
 constexpr int kSplitN = 96;         // tails per accumulator tile
 
 // (p-1)^(t-1) coefficient vectors per tail subset.
@@ -154,60 +156,69 @@ FPK_HD bool tail_next(Tail &a, int k, int t, int b) {
   return true;
 }
 
-// Stems: `m` = q, Q = the other l - 1 rows, d = the packed counter digits of
-// all l coefficients (slot l - 1: row q), qi the rank of Q, ci the counter
-// (kept only for b > 2; for b = 2 the digits are the counter).  ncl =
-// (b/2) b^(l-1) coefficient vectors per row subset.
+// A stem: its largest row, the mask of the other l - 1 rows, and the packed
+// counter digits of all l coefficients (slot l - 1: the largest row).  The
+// next stem follows from these alone (no ranks are kept: a lane of the
+// kernel holds its stem in few registers).
+struct StemPos {
+  int m;
+  uint64_t Q, d;
+};
+
+// Stem of index J; ncl = (b/2) b^(l-1) coefficient vectors per row subset.
 template <int DB, class BT>
-FPK_HD fpenum::Prefix stem_unrank(const BT &B, uint64_t J, int k, int t, int l, int b, uint64_t ncl, uint64_t *ci) {
-  fpenum::Prefix P;
+FPK_HD StemPos stem_unrank(const BT &B, uint64_t J, int k, int t, int l, int b, uint64_t ncl) {
+  StemPos P;
   P.m = comb_floor(B, l - 1, k - t - 1, l, ncl, J);
   const uint64_t rem = J - ncl * B(P.m, l);
+  uint64_t qi, ci;
   if constexpr (DB == 1) {
-    P.qi = rem >> (l - 1);
-    *ci = rem & (ncl - 1);
+    qi = rem >> (l - 1);
+    ci = rem & (ncl - 1);
   } else if ((rem | ncl) >> 32) {
-    P.qi = rem / ncl;
-    *ci = rem - P.qi * ncl;
+    qi = rem / ncl;
+    ci = rem - qi * ncl;
   } else {
-    P.qi = (uint32_t)rem / (uint32_t)ncl;
-    *ci = (uint32_t)rem - (uint32_t)P.qi * (uint32_t)ncl;
+    qi = (uint32_t)rem / (uint32_t)ncl;
+    ci = (uint32_t)rem - (uint32_t)qi * (uint32_t)ncl;
   }
-  P.Q = fpenum::rd_unrank(B, P.qi, P.m, l - 1);
+  P.Q = fpenum::rd_unrank(B, qi, P.m, l - 1);
   if constexpr (DB == 1) {
-    P.d = *ci;
+    P.d = ci;
+  } else if (ci >> 32) {
+    P.d = fpenum::counter_digits<DB>(ci, b, l);
   } else {
-    P.d = fpenum::counter_digits<DB>(*ci, b, l);
+    P.d = 0;
+    uint32_t c = (uint32_t)ci;
+    for (int s = 0; s < l; ++s) {
+      P.d |= (uint64_t)(c % (uint32_t)b) << (s * DB);
+      c /= (uint32_t)b;
+    }
   }
   return P;
 }
 
+// The last counter value of a row subset: digits b - 1, the top one b/2 - 1.
+template <int DB>
+FPK_HD uint64_t stem_last(int b, int l) {
+  const int top = DB * (l - 1);
+  const uint64_t all = DB == 1 ? ~0ull : 0x1111111111111111ull * (uint64_t)(b - 1);
+  return (all & fpenum::low_mask(top)) | (uint64_t)(b / 2 - 1) << top;
+}
+
 // Next stem: the slot whose coefficient changed by *dir, or -1 when the row
-// subset changed (all coefficients back to 1).  nq: subsets C(m, l - 1).
-template <int DB, class BT>
-FPK_HD int stem_advance(const BT &B, fpenum::Prefix &P, uint64_t &ci, uint64_t &nq, uint64_t ncl, int b, int l,
-                        int *dir) {
-  if constexpr (DB == 1) {
-    if (P.d + 1 < ncl) return fpenum::gray_step<1>(&P.d, b, l, dir);
-  } else {
-    if (ci + 1 < ncl) {
-      ++ci;
-      return fpenum::gray_step<DB>(&P.d, b, l, dir);
-    }
-  }
-  ci = 0;
+// subset changed (all coefficients back to 1).
+template <int DB>
+FPK_HD int stem_advance(StemPos &P, int b, int l, int *dir) {
+  if (P.d != stem_last<DB>(b, l)) return fpenum::gray_step<DB>(&P.d, b, l, dir);
   P.d = 0;
-  if (P.qi + 1 < nq) {
-    uint64_t nQ = P.Q;
-    int rm = 0, ad = 0;
-    fpenum::rd_next(P.Q, P.m, l - 1, &nQ, &rm, &ad);
+  uint64_t nQ = P.Q;
+  int rm = 0, ad = 0;
+  if (fpenum::rd_next(P.Q, P.m, l - 1, &nQ, &rm, &ad)) {
     P.Q = nQ;
-    ++P.qi;
   } else {
     ++P.m;
-    P.qi = 0;
     P.Q = fpenum::low_mask(l - 1);
-    nq = B(P.m, l - 1);
   }
   return -1;
 }
@@ -217,7 +228,7 @@ FPK_HD int stem_advance(const BT &B, fpenum::Prefix &P, uint64_t &ci, uint64_t &
 // index and pair entry; false: prefix index, leaf row and coefficient).
 template <int DB, class BT>
 FPK_HD uint64_t split_key(const BT &B, bool pair, int k, int p, int g, uint32_t pass, uint32_t weight,
-                          const fpenum::Prefix &P, int l, const Tail &a, int sign) {
+                          const StemPos &P, int l, const Tail &a, int sign) {
   const int b = p - 1;
   int row[fpenum::kBinomCols], c[fpenum::kBinomCols];
   int n = 0;

@@ -31,10 +31,10 @@
 
 namespace fpk {
 
-constexpr int kSplitGroups = kSplitThreads / kSplitGroup;
 constexpr int kSplitWarps = kSplitThreads / 32;
-constexpr uint32_t kTmemCols = 512;   // all of the SM's tensor memory: one such CTA per SM
-constexpr uint32_t kTmemD = 32;       // a warpgroup's columns: the A tile (up to 32), then the results
+constexpr uint32_t kTmemCols = 512;    // all of the SM's tensor memory: one such CTA per SM
+constexpr uint32_t kTmemGroup = 128;   // a warpgroup's columns: the A tile (up to 32), then the results
+constexpr uint32_t kTmemD = 32;
 
 // ------------------------------------------------------------- tcgen05 ----
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -257,6 +257,10 @@ struct SplitShared {
                                   // of its task (two, since the first warp may be a product ahead of the last)
   unsigned long long best_key;    // the code's best key (inverted) and finished flag, as the scheduler last read them
   int32_t finished;
+  int32_t failed;                 // a product never came: no more are issued
+  SlotState *states;              // of the launch
+  SlotAux *aux;
+  CtlDyn *cdyn;
   SplitQueue queue[kSplitWarps];
   SplitTask task[2];              // the one that runs and the next one
   // mbarriers: of each task buffer, full (1 arrival), near its end (one per
@@ -268,41 +272,34 @@ struct SplitShared {
 template <int RW>
 struct Stem {
   uint32_t s[RW];
-  fpenum::Prefix pf;
-  uint64_t ci, nq, qrows;
+  StemPos pos;
 };
 
 template <int P, int R, int W, int DB>
 __device__ __forceinline__ void stem_sum(Stem<R * W> &x, const uint32_t *mult, int l) {
   constexpr int b = P - 1;
-  set_row<P, R, W>(x.s, mult, x.pf.m, fpenum::gray_digit<DB>(x.pf.d, l - 1, b, l) + 1, P);
-  uint64_t Q = x.pf.Q;
-  x.qrows = 0;
+  set_row<P, R, W>(x.s, mult, x.pos.m, fpenum::gray_digit<DB>(x.pos.d, l - 1, b, l) + 1, P);
+  uint64_t Q = x.pos.Q;
   for (int s = 0; s + 1 < l; ++s) {
     const int q = fpenum::ctz64(Q);
     Q &= Q - 1;
-    if (s < kSlotRows) x.qrows |= (uint64_t)q << (6 * s);
-    add_row<P, R, W>(x.s, mult, q, fpenum::gray_digit<DB>(x.pf.d, s, b, l) + 1, P);
+    add_row<P, R, W>(x.s, mult, q, fpenum::gray_digit<DB>(x.pos.d, s, b, l) + 1, P);
   }
 }
 
 template <int P, int R, int W, int DB>
 __device__ __forceinline__ void stem_start(Stem<R * W> &x, const uint32_t *mult, const fpenum::BinomCols &B,
                                            uint64_t J, int k, int t, int l, uint64_t ncl) {
-  x.pf = stem_unrank<DB>(B, J, k, t, l, P - 1, ncl, &x.ci);
-  x.nq = B(x.pf.m, l - 1);
+  x.pos = stem_unrank<DB>(B, J, k, t, l, P - 1, ncl);
   stem_sum<P, R, W, DB>(x, mult, l);
 }
 
 template <int P, int R, int W, int DB>
-__device__ __forceinline__ void stem_next(Stem<R * W> &x, const uint32_t *mult, const fpenum::BinomCols &B, int l,
-                                          uint64_t ncl) {
+__device__ __forceinline__ void stem_next(Stem<R * W> &x, const uint32_t *mult, int l) {
   int dir = 1;
-  const int slot = stem_advance<DB>(B, x.pf, x.ci, x.nq, ncl, P - 1, l, &dir);
+  const int slot = stem_advance<DB>(x.pos, P - 1, l, &dir);
   if (slot >= 0) {
-    const int q = slot == l - 1          ? x.pf.m
-                  : slot < kSlotRows     ? (int)(x.qrows >> (6 * slot)) & 63
-                                         : fpenum::nth_member(x.pf.Q, slot);
+    const int q = slot == l - 1 ? x.pos.m : fpenum::nth_member(x.pos.Q, slot);
     add_row<P, R, W>(x.s, mult, q, dir > 0 ? 1 : P - 1, P);  // c -> c+1: +A; c -> c-1: +(p-1)A
   } else {
     stem_sum<P, R, W, DB>(x, mult, l);
@@ -332,7 +329,7 @@ __device__ __forceinline__ void split_weights(const uint32_t (&s)[R * W], const 
 // under the bound only.
 template <int DB>
 __device__ __noinline__ uint64_t hit_key(const fpenum::BinomCols B, bool pair, int k, int p, int g, int pass, int wp,
-                                         int wm, int thr, fpenum::Prefix pf, int l, uint32_t tail) {
+                                         int wm, int thr, StemPos pf, int l, uint32_t tail) {
   const Tail a = tail_unpack(tail);
   uint64_t best = kNoKey;
   if (wp < thr) best = split_key<DB>(B, pair, k, p, g, (uint32_t)pass, (uint32_t)(g + wp), pf, l, a, 0);
@@ -346,25 +343,27 @@ __device__ __noinline__ uint64_t hit_key(const fpenum::BinomCols B, bool pair, i
 // 2 or 4 interleaved slices of the tails, so nothing is handed out inside a
 // task; `near` is told when its last step begins.
 template <int P, int R, int W>
-__device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &cl, const uint32_t *mult,
-                           const uint32_t *tails, uint32_t table, uint32_t tmem, uint32_t mbar, uint32_t &parity,
-                           uint32_t near, const fpenum::BinomCols &B, SplitShared &sh, SlotState *st, SlotAux *ax,
-                           CtlDyn *cd, unsigned long long &count) {
+__device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, SplitShared &sh, int buf, const uint32_t *mult,
+                                                         const uint32_t *tails, uint32_t table, uint32_t tmem,
+                                                         uint32_t &parity, const fpenum::BinomCols &B) {
+  const PassDesc &pd = sh.task[buf].pd;
+  const Claim &cl = sh.task[buf].cl;
   constexpr int DB = P == 3 ? 1 : 4, RW = R * W, b = P - 1;
   constexpr unsigned FULL = 0xffffffffu;
-  const int k = sd.k, g = pd.g, t = pd.tail_rows, l = g - t, pass = cl.pass;
+  const int k = sd.k, g = pd.g, t = pd.tail_rows, l = g - t;
   const int lane = threadIdx.x & 31, row = threadIdx.x & (kSplitGroup - 1);
   const int warp = __shfl_sync(FULL, (int)(threadIdx.x >> 5), 0), grp = warp / (kSplitGroup / 32);
+  const uint32_t mbar = smem_u32(&sh.product[grp]), near = smem_u32(&sh.near[buf]);
   const bool pair = sd.pair_sigp > 0;
   const uint64_t ncl = pd.ncl;
   const uint32_t etot = tails_above(B, k, t, b, -1);
   const uint32_t first = cl.block * pd.block, nb = min(pd.block, etot - first);
   const uint64_t ns = l > 0 ? B(cl.zhi, l) * ncl : 1ull;
   const int K = sd.split_k, nu = sd.split_nu;
-  const unsigned long long cpe = l > 0 ? 2ull : 1ull;  // codewords per stem and tail
+  uint32_t seen = 0;  // this lane's stem-tail pairs (a task's fit 32 bits): two codewords each, or one (l = 0)
   // the warpgroup's units [u0, u0 + steps) and its slice of the tails
-  const uint32_t parts = (uint32_t)kSplitGroups >> pd.esplit, part = (uint32_t)grp >> pd.esplit;
-  const uint32_t slices = 1u << pd.esplit, slice = (uint32_t)grp & (slices - 1u);
+  const uint32_t parts = pd.esplit ? 1u : (uint32_t)kSplitGroups, part = pd.esplit ? 0u : (uint32_t)grp;
+  const uint32_t slices = pd.esplit ? (uint32_t)kSplitGroups : 1u, slice = pd.esplit ? (uint32_t)grp : 0u;
   const uint32_t share = ((uint32_t)(cl.uhi - cl.ulo) + parts - 1) / parts;
   const uint64_t u0 = min(cl.ulo + (uint64_t)part * share, cl.uhi);
   const uint32_t steps = (uint32_t)(min(u0 + share, cl.uhi) - u0);
@@ -388,17 +387,14 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
     if (__any_sync(FULL, best != kNoKey)) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) best = min(best, (uint64_t)__shfl_xor_sync(FULL, (unsigned long long)best, o));
-      if (lane == 0) record(st, ax, pass, best);
+      if (lane == 0) record(sh.states, sh.aux, cl.pass, best);
       thr = min(thr, (int)key_weight(best) - g + 1);
     }
   };
   Stem<RW> x;
 #pragma unroll
   for (int q = 0; q < RW; ++q) x.s[q] = 0;
-  x.pf = fpenum::Prefix{-1, 0, 0, 0};
-  x.ci = 0;
-  x.nq = 1;
-  x.qrows = 0;
+  x.pos = StemPos{-1, 0, 0};
 
   if (pd.direct) {
     // few codewords: one stem per warpgroup at a time, its tails over the 128
@@ -407,8 +403,8 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
     nearly();
     if (l > 0 && steps) stem_start<P, R, W, DB>(x, mult, B, u0, k, t, l, ncl);
     for (uint32_t i = 0; i < steps && !finished(); ++i) {
-      if (l > 0 && i) stem_next<P, R, W, DB>(x, mult, B, l, ncl);
-      const uint32_t E = min(nb, tails_above(B, k, t, b, x.pf.m) - first);
+      if (l > 0 && i) stem_next<P, R, W, DB>(x, mult, l);
+      const uint32_t E = min(nb, tails_above(B, k, t, b, x.pos.m) - first);
       take_up();
       for (uint32_t e0 = slice * kSplitGroup; e0 < E; e0 += kSplitGroup * slices) {
         const uint32_t e = e0 + row;
@@ -418,27 +414,26 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
           int wp, wm;
           split_weights<P, R, W>(x.s, tail_unpack(tl), mult, wp, wm);
           if (wp < thr || (l > 0 && wm < thr))
-            best = hit_key<DB>(B, pair, k, P, g, pass, wp, wm, thr, x.pf, l, tl);
-          count += cpe;
+            best = hit_key<DB>(B, pair, k, P, g, cl.pass, wp, wm, thr, x.pos, l, tl);
+          ++seen;
         }
         note(best);
       }
     }
-    return;
+    return (unsigned long long)seen << (l > 0 ? 1 : 0);
   }
 
-  const uint32_t tA = tmem + (uint32_t)grp * (kTmemCols / kSplitGroups), tD = tA + kTmemD;
+  const uint32_t tA = tmem + (uint32_t)grp * kTmemGroup, tD = tA + kTmemD;
   const uint32_t my_lanes = (uint32_t)(warp & 3) << 21;  // 32 lanes a warp, in the address's upper half
-  bool dead = false;
   const uint64_t J0 = u0 * kSplitGroup, J = J0 + (uint64_t)row * steps;  // a lane's run of stems
   const uint32_t nst = J < ns ? (uint32_t)min((uint64_t)steps, ns - J) : 0u;
   if (l > 0 && nst) stem_start<P, R, W, DB>(x, mult, B, J, k, t, l, ncl);
   // tails of the block above the run's first stem: as many tiles as any lane needs
   const int q0 = l > 0 && steps ? comb_floor(B, l - 1, k - t - 1, l, ncl, J0) : -1;
   const uint32_t tiles = (min(nb, tails_above(B, k, t, b, q0) - first) + kSplitN - 1) / kSplitN;
-  if (steps == 0 || slice >= tiles) {  // the same for the whole warpgroup
+  if (steps == 0 || slice >= tiles || *(volatile int32_t *)&sh.failed) {  // the same for the whole warpgroup
     nearly();
-    return;
+    return 0;
   }
   for (uint32_t i = 0; i < steps; ++i) {
     if (i + 1 == steps) nearly();
@@ -459,6 +454,7 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
       tmem_wait_store();
     }
     uint32_t n = 0;  // candidates in the warp's queue
+    int thr_set = thr;  // the threshold in the rows' last words
     // exact weights of `cnt` candidates from `at`: a lane takes one and fetches the owner's stem
     auto check = [&](uint32_t at, uint32_t cnt) {
       __syncwarp();
@@ -468,19 +464,18 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
       uint32_t so[RW];
 #pragma unroll
       for (int q = 0; q < RW; ++q) so[q] = __shfl_sync(FULL, x.s[q], src);
-      const int qo = __shfl_sync(FULL, x.pf.m, src);
+      const int qo = __shfl_sync(FULL, x.pos.m, src);
       const uint32_t tl = tails[item_ >> 5];
       const Tail a = tail_unpack(tl);
       int wp = 1 << 20, wm = 1 << 20;
       if (have && a.z > qo) split_weights<P, R, W>(so, a, mult, wp, wm);
       const bool hit = wp < thr || (l > 0 && wm < thr);
       if (__any_sync(FULL, hit)) {
-        fpenum::Prefix po;
+        StemPos po;
         po.m = qo;
-        po.qi = 0;
-        po.Q = __shfl_sync(FULL, (unsigned long long)x.pf.Q, src);
-        po.d = __shfl_sync(FULL, (unsigned long long)x.pf.d, src);
-        note(hit ? hit_key<DB>(B, pair, k, P, g, pass, wp, wm, thr, po, l, tl) : kNoKey);
+        po.Q = __shfl_sync(FULL, (unsigned long long)x.pos.Q, src);
+        po.d = __shfl_sync(FULL, (unsigned long long)x.pos.d, src);
+        note(hit ? hit_key<DB>(B, pair, k, P, g, cl.pass, wp, wm, thr, po, l, tl) : kNoKey);
       }
       __syncwarp();
     };
@@ -534,11 +529,11 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
       } else {
         group_arrive(1 + grp);
       }
-      if (!dead && !mbar_wait(mbar, parity)) {
-        dead = true;  // never seen: reported as a timeout, and the rest of the launch drains without results
-        atomicExch(&cd->err, 1);
+      if (!__all_sync(FULL, mbar_wait(mbar, parity))) {  // never seen: reported as a timeout; nothing more is issued
+        *(volatile int32_t *)&sh.failed = 1;
+        atomicExch(&sh.cdyn->err, 1);
+        return 0;
       }
-      __syncwarp();
       stop = *(volatile int32_t *)&sh.stop[grp][parity];
       parity ^= 1u;
       tc_after_sync();
@@ -554,24 +549,36 @@ __device__ void task_split(const SlotDesc &sd, const PassDesc &pd, const Claim &
         a1 = and3(a1, v1[q], v1[q + 1]);
         a2 = and3(a2, v2[q], v2[q + 1]);
       }
-      if (__any_sync(FULL, (~and3(a0, a1, a2) & 0x80008000u) != 0)) scan(v0, v1, v2, c * kSplitN);
+      if (__any_sync(FULL, (~and3(a0, a1, a2) & 0x80008000u) != 0)) {
+        scan(v0, v1, v2, c * kSplitN);
+        take_up();
+        if (thr < thr_set && c + slices < tiles) {  // a lower bound since: into the rows, for the step's other tiles
+          thr_set = thr;
+          const uint32_t marks = act ? stem_marks<P>(nu, thr) : kStemNone;
+          __syncwarp();
+          asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(tA + my_lanes + (uint32_t)(K / 4 - 1)), "r"(marks)
+                       : "memory");
+          tmem_wait_store();
+        }
+      }
     }
     if (n) check(0, n);
     if (act) {
       // this lane's tails, in the slice's tiles
-      const uint32_t above = tails_above(B, k, t, b, x.pf.m);
+      const uint32_t above = tails_above(B, k, t, b, x.pos.m);
       const uint32_t E = above > first ? min(nb, above - first) : 0u;
       const uint32_t full = E / kSplitN, rest = E - full * kSplitN;  // whole tiles, then part of one
-      const uint32_t mine = full > slice ? (full - slice + slices - 1) >> pd.esplit : 0u;
-      const uint32_t tailn = mine * kSplitN + ((full & (slices - 1)) == slice ? rest : 0u);
-      count += tailn * cpe;
+      const uint32_t mine = full > slice ? (full - slice + slices - 1) / slices : 0u;
+      const uint32_t tailn = mine * kSplitN + (full % slices == slice ? rest : 0u);
+      seen += tailn;
     }
     if (stop) {
       if (i + 1 < steps) nearly();
       break;
     }
-    if (i + 1 < nst) stem_next<P, R, W, DB>(x, mult, B, l, ncl);
+    if (i + 1 < nst) stem_next<P, R, W, DB>(x, mult, l);
   }
+  return (unsigned long long)seen << (l > 0 ? 1 : 0);
 }
 
 // Waits bounded by time (globaltimer looked at now and then).
@@ -598,17 +605,17 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 5, 512;" ::: "memory"); }
+__device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 5, %0;" ::"n"(kSplitThreads) : "memory"); }
 
 // The kernel: claims, counts and termination tests follow bz_kernel's
-// protocol on the same state.  One code per launch.  Sixteen warps work;
-// the seventeenth claims: it hands out the next task when the running one
+// protocol on the same state.  One code per launch.  Sixteen warps work; one
+// more claims: it hands out the next task when the running one
 // nears its end and counts the finished one off while the next runs (in
 // bz_kernel, where thread 0 does both between tasks, a hand-off holds the
 // CTA for about 4 us, a tenth to a third of these searches).  Claiming only
 // near the end keeps the tasks of a pass's end with the CTAs that are free.
 template <int P, int R, int W>
-__global__ void __launch_bounds__(kSplitThreads + 32, 1)
+__global__ void __launch_bounds__(kSplitLaunch, 1)
     split_kernel(const SlotDesc *__restrict__ slots, SlotState *states, const CtlStatic *__restrict__ ctl, CtlDyn *cdyn,
                  KParams kp) {
   extern __shared__ uint4 smem_raw[];
@@ -621,7 +628,7 @@ __global__ void __launch_bounds__(kSplitThreads + 32, 1)
   __shared__ uint32_t s_tmem;
 
   const CtlStatic cs = *ctl;
-  const int tid = threadIdx.x, threads = kSplitThreads + 32;
+  const int tid = threadIdx.x, threads = kSplitLaunch;
   const unsigned long long t_start = globaltimer();
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   // longest wait for another warp: past every bounded wait of the claims
@@ -639,8 +646,12 @@ __global__ void __launch_bounds__(kSplitThreads + 32, 1)
       mbar_init(smem_u32(&s_sh.done[i]), kSplitWarps);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_sh.failed = 0;
     s_sh.best_key = 0;
     s_sh.finished = 0;
+    s_sh.states = states;
+    s_sh.aux = cs.aux;
+    s_sh.cdyn = cdyn;
     s_cc.sd = load_nc(&slots[0]);  // one thread per CTA, through L1: every CTA reads the same bytes at once
     s_cc.slot = 0;
     s_cc.gen = s_cc.sd.seq & kGenMask;
@@ -679,8 +690,9 @@ __global__ void __launch_bounds__(kSplitThreads + 32, 1)
     }
   }
   __syncthreads();
-  if (warp == kSplitWarps) {
-    if ((tid & 31) == 0) {
+  if (warp >= kSplitWarps) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+    if (tid == kSplitThreads) {
       // what the tables hold: the set, the block (tail length and size, index) and how much of it
       int rr = 0, staged_j = -1, built = -1, built_n = 0;
       unsigned int built_block = 0;
@@ -753,6 +765,8 @@ __global__ void __launch_bounds__(kSplitThreads + 32, 1)
         } else if (globaltimer() - since > wait_ns) {
           atomicExch(&cdyn->err, 1);  // a warp never finished: report a timeout
           break;
+        } else {
+          __nanosleep(200);  // the issue slots belong to the warps that work
         }
       }
       s_sh.task[head & 1u].cmd = kCmdExit;
@@ -760,15 +774,15 @@ __global__ void __launch_bounds__(kSplitThreads + 32, 1)
     }
     __syncwarp();
   } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
     const SlotDesc &sd = s_cc.sd;
-    const int K = sd.split_k;
     uint32_t *mult = reinterpret_cast<uint32_t *>(smem + kBinomBytes);
     uint32_t *tails = reinterpret_cast<uint32_t *>(smem + split_off_tails(sd.k, P, sd.rwpad));
     char *table = smem + split_off_table(sd.k, P, sd.rwpad, sd.split_cap);
-    const int grp = warp / (kSplitGroup / 32);
     uint32_t parity = 0;
     for (uint32_t n = 0;; ++n) {
-      SplitTask &tk = s_sh.task[n & 1u];
+      const int b = (int)(n & 1u);
+      SplitTask &tk = s_sh.task[b];
       if (!mbar_wait_ns(smem_u32(&s_sh.full[n & 1u]), (n >> 1) & 1u, wait_ns)) {
         atomicExch(&cdyn->err, 1);
         break;
@@ -786,26 +800,24 @@ __global__ void __launch_bounds__(kSplitThreads + 32, 1)
         }
         if (tk.build && !tk.drop) {
           const uint32_t etot = tails_above(binom, sd.k, tk.pd.tail_rows, P - 1, -1), first = tk.cl.block * tk.pd.block;
-          build_tails<P, R, W>(tails, table, mult, binom, sd.k, tk.pd.tail_rows, first, min(tk.pd.block, etot - first), K,
-                               sd.split_nu, tk.build == 2);
+          build_tails<P, R, W>(tails, table, mult, binom, sd.k, tk.pd.tail_rows, first, min(tk.pd.block, etot - first),
+                               sd.split_k, sd.split_nu, tk.build == 2);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the tensor cores read the table
           workers_sync();
         }
       }
       unsigned long long count = 0;
-      const uint32_t near = smem_u32(&s_sh.near[n & 1u]);
       if (tk.cl.skip || tk.drop || tk.pd.g == 1) {
-        if ((tid & (kSplitGroup - 1)) == 0) mbar_arrive(near);
+        if ((tid & (kSplitGroup - 1)) == 0) mbar_arrive(smem_u32(&s_sh.near[b]));
         if (!tk.cl.skip && !tk.drop && tk.cl.ulo == 0) task_rows<P, R, W>(sd, tk.cl.pass, mult, tk.cl.U, &states[0], cs.aux, count);
       } else {
-        task_split<P, R, W>(sd, tk.pd, tk.cl, mult, tails, smem_u32(table), tmem, smem_u32(&s_sh.product[grp]), parity, near,
-                            binom, s_sh, &states[0], cs.aux, cdyn, count);
+        count = task_split<P, R, W>(sd, s_sh, b, mult, tails, smem_u32(table), tmem, parity, binom);
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
       if ((tid & 31) == 0) {
         if (count) atomicAdd(&tk.count, count);
-        mbar_arrive(smem_u32(&s_sh.done[n & 1u]));
+        mbar_arrive(smem_u32(&s_sh.done[b]));
       }
     }
   }

@@ -63,7 +63,7 @@ struct PassDesc {
   uint32_t block;          // tails per block
   uint8_t tail_rows;       // rows of a tail (2 or 3)
   uint8_t direct;          // 1: few codewords, every weight exact
-  uint8_t esplit;          // log2 of the warpgroups that share a task's stems and split its tails
+  uint8_t esplit;          // 1: a CTA's warpgroups share a task's stems and split its tails
   uint8_t pad0;
 };
 

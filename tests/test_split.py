@@ -36,7 +36,7 @@ def test_split_pass_visits_each_class_once(p, n, k, pair, lib):
             continue
         walks = [dict(ctas=152), dict(ctas=3)]
         walks += [dict(tail_rows=t, block=bl, unit=u, esplit=s) for t in (2, 3) if t <= g
-                  for bl, u, s in ((96, 1, 0), (192, 4, 1), (7 * 96, 3, 2))]
+                  for bl, u, s in ((96, 1, 0), (192, 4, 1), (7 * 96, 6, 0))]
         for w in walks:
             keys = B.fpcode_test_split_pass(pr, i, **w)
             assert keys is not None and len(keys) == size == math.comb(k, g) * (p - 1) ** (g - 1), (g, w)
