@@ -237,11 +237,7 @@ void fill_static(const Layout &L, const std::vector<const fph::Prepared *> &code
     sd.pair_sigp = P.pair ? P.pair_sigp : 0;
     sd.pair_quick_max = P.pair_quick_max;
     sd.nsegs = (int)(P.split ? P.split_segs.size() : P.segs.size());
-    if (P.split) {
-      sd.split_k = P.split_k;
-      sd.split_nu = P.split_nu;
-      sd.split_cap = P.split_cap;
-    }
+    if (P.split) sd.set_split(P.split_k, P.split_nu, P.split_cap);
     sd.table = reinterpret_cast<const uint32_t *>(d + L.table_off[i]);
     sd.passes = reinterpret_cast<const PassDesc *>(d + L.pass_off[i]);
     std::memcpy(h + L.off_slots + i * sizeof(SlotDesc), &sd, sizeof(sd));
@@ -733,10 +729,11 @@ int fpcode_min_distance_batch(int num, const fpcode_desc *codes, void *stream, c
       if (preps[i]->variant < 12 && !per_variant) (preps[i]->W <= narrow_w ? narrow : wide).push_back(i);
       else other[preps[i]->variant].push_back(i);
     }
-    if (!narrow.empty()) groups.push_back(narrow);
-    if (!wide.empty()) groups.push_back(wide);
+    // the kernels of single variants first: few codes, long tails
     for (auto &g : other)
       if (!g.empty()) groups.push_back(g);
+    if (!narrow.empty()) groups.push_back(narrow);
+    if (!wide.empty()) groups.push_back(wide);
   }
   std::vector<size_t> woff(num + 1, 0);
   for (int i = 0; i < num; ++i) woff[i + 1] = woff[i] + (size_t)codes[i].n;
@@ -787,29 +784,46 @@ int fpcode_min_distance_batch(int num, const fpcode_desc *codes, void *stream, c
   }
   s = ws_reserve(*c, std::max<size_t>(dev_total, 256), std::max<size_t>(pin_total, 256));
   if (s) return s;
+  // The launches are independent: the first runs on the caller's stream, the
+  // others on side streams between a fork and a join, so that one kernel's
+  // CTAs fill the SMs that the last tasks of another have left (one after
+  // another, each launch's tail left most SMs idle).  The copies and resets
+  // go first, since a reset is a kernel and would wait for a free SM.
   int err = FPCODE_OK;
+  cudaEvent_t fork = nullptr;
+  auto ok = [&](cudaError_t e) {
+    if (e != cudaSuccess && !err) err = FPCODE_ECUDA;
+    return !err;
+  };
   for (auto &g : ls) {
     char *d = c->ws + g.dev_off;
     fill_static(g.L, g.codesv, *c, c->ws_pinned + g.pin_off, d, 0);
-    if (cudaEventCreate(&g.e0) != cudaSuccess || cudaEventCreate(&g.e1) != cudaSuccess) {
-      err = FPCODE_ECUDA;
+    if (!ok(cudaEventCreate(&g.e0)) || !ok(cudaEventCreate(&g.e1)) ||
+        !ok(cudaMemcpyAsync(d, c->ws_pinned + g.pin_off, g.L.static_bytes, cudaMemcpyHostToDevice, st)) ||
+        !ok(cudaMemsetAsync(d + g.L.off_states, 0, g.L.dyn_bytes + g.L.aux_bytes, st)))
       break;
-    }
-    if (cudaMemcpyAsync(d, c->ws_pinned + g.pin_off, g.L.static_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-        cudaMemsetAsync(d + g.L.off_states, 0, g.L.dyn_bytes + g.L.aux_bytes, st) != cudaSuccess ||
-        cudaEventRecord(g.e0, st) != cudaSuccess) {
-      err = FPCODE_ECUDA;
-      break;
-    }
-    if ((err = launch(g.fn, g.ctas, g.smem, st, d, g.L, kparams(o, 0))) != FPCODE_OK) break;
-    if (cudaEventRecord(g.e1, st) != cudaSuccess ||
-        cudaMemcpyAsync(c->ws_pinned + g.rb_off, d + g.L.off_states, g.L.dyn_bytes, cudaMemcpyDeviceToHost, st) !=
-            cudaSuccess) {
-      err = FPCODE_ECUDA;
-      break;
-    }
   }
-  if (!err && cudaStreamSynchronize(st) != cudaSuccess) err = FPCODE_ECUDA;
+  if (!err && ls.size() > 1 && ok(cudaEventCreateWithFlags(&fork, cudaEventDisableTiming))) {
+    for (auto &side : c->side)
+      if (!side && ok(cudaStreamCreateWithFlags((cudaStream_t *)&side, cudaStreamNonBlocking)) == false) break;
+    ok(cudaEventRecord(fork, st));
+  }
+  for (size_t li = 0; li < ls.size() && !err; ++li) {
+    Launch &g = ls[li];
+    char *d = c->ws + g.dev_off;
+    cudaStream_t sl = li == 0 ? st : (cudaStream_t)c->side[(li - 1) % DevCtx::kSide];
+    if (li > 0 && !ok(cudaStreamWaitEvent(sl, fork, 0))) break;
+    if (!ok(cudaEventRecord(g.e0, sl))) break;
+    if ((err = launch(g.fn, g.ctas, g.smem, sl, d, g.L, kparams(o, 0))) != FPCODE_OK) break;
+    if (!ok(cudaEventRecord(g.e1, sl)) ||
+        !ok(cudaMemcpyAsync(c->ws_pinned + g.rb_off, d + g.L.off_states, g.L.dyn_bytes, cudaMemcpyDeviceToHost, sl)))
+      break;
+  }
+  // everything has ended before the workspace is handed back, also after an error
+  for (size_t li = 1; li < ls.size() && li <= (size_t)DevCtx::kSide; ++li)
+    if (c->side[li - 1]) ok(cudaStreamSynchronize((cudaStream_t)c->side[li - 1]));
+  ok(cudaStreamSynchronize(st));
+  if (fork) cudaEventDestroy(fork);
   int nlaunch = -1;
   for (auto &g : ls) {
     if (!err && g.e1) {

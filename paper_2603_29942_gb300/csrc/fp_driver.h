@@ -22,6 +22,9 @@ struct DevCtx {
   char *ws_pinned = nullptr;
   size_t ws_pinned_bytes = 0;
   void *ev0 = nullptr, *ev1 = nullptr;  // cudaEvent_t around the kernel of a workspace search
+  // batches: streams of the launches after the first (guarded by ws_mu, made once)
+  static constexpr int kSide = 3;
+  void *side[kSide] = {nullptr, nullptr, nullptr};
 };
 
 // Context of the current device (created on first use).

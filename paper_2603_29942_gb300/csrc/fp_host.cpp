@@ -837,17 +837,9 @@ void plan_split(Prepared *P, int ctas) {
                            cut_tails(*P, 3, std::max<uint32_t>(fpk::kSplitN, cap / 2 / fpk::kSplitN * fpk::kSplitN))};
   P->split_segs.clear();
   for (auto &d : P->passes) {
-    d.phases = 0;
-    d.plan_ctas = (uint32_t)ctas;
-    d.unit = 1;
-    d.pl = 0;
     d.seg_off = (uint32_t)P->split_segs.size();
     d.nseg = 0;
-    d.direct = 0;
-    d.esplit = 0;
-    d.tail_rows = 0;
-    d.block = 0;
-    d.ncl = 1;
+    d.set_split(0, false, false, 0, 1);
     if (d.g == 1) {
       d.ntasks = 1;
       continue;
@@ -859,12 +851,13 @@ void plan_split(Prepared *P, int ctas) {
       return v;
     };
     int t = 2;
+    bool direct = false, esplit = false;
     uint32_t nb = 0;
     double total = 0;
     const TailCut *cut = nullptr;
     const uint64_t combos = g == 2 ? d.size : d.size / 2;
     if (combos <= kDirectPairs) {
-      d.direct = 1;
+      direct = true;
       nb = fpk::tails_above(binom(), k, 2, b, -1);
     } else {
       double best = 0;
@@ -884,9 +877,7 @@ void plan_split(Prepared *P, int ctas) {
       nb = cut->nb;
     }
     const int l = g - t;
-    d.tail_rows = (uint8_t)t;
-    d.block = nb;
-    d.ncl = ncl_of(l);
+    const uint64_t ncl = ncl_of(l);
     uint32_t tasks = 0;
     auto add = [&](uint32_t item0, uint32_t item1, uint64_t per, uint32_t block, int zhi) {
       if (item0 >= item1) return;
@@ -901,16 +892,16 @@ void plan_split(Prepared *P, int ctas) {
       s.zhi = (uint8_t)zhi;
       P->split_segs.push_back(s);
     };
-    if (d.direct) {
+    if (direct) {
       // runs of stems with about the same number of tails, as many to a task
       // as give every warpgroup of the grid the same work
-      d.esplit = g == 2 ? 1 : 0;
+      esplit = g == 2;
       auto stem_clocks = [&](int q) {
         return 400.0 + 800.0 * (double)((fpk::tails_above(binom(), k, t, b, q) + fpk::kSplitGroup - 1) / fpk::kSplitGroup);
       };
       double work = 0;
-      for (int q = std::max(l - 1, 0); l > 0 && q < k - 2; ++q) work += (double)(binom().c[q][l - 1] * d.ncl) * stem_clocks(q);
-      const uint32_t items = (uint32_t)(l > 0 ? binom().c[k - 2][l] * d.ncl : 1);
+      for (int q = std::max(l - 1, 0); l > 0 && q < k - 2; ++q) work += (double)(binom().c[q][l - 1] * ncl) * stem_clocks(q);
+      const uint32_t items = (uint32_t)(l > 0 ? binom().c[k - 2][l] * ncl : 1);
       // the passes of one level run side by side, one per information set
       const double target = std::max(3000.0, work * std::min(P->m, 4) / (fpk::kSplitGroups * C));
       uint32_t at = 0;
@@ -918,7 +909,7 @@ void plan_split(Prepared *P, int ctas) {
         const double c = stem_clocks(l > 0 ? q : -1);
         int q1 = q + 1;
         while (l > 0 && q1 < k - 2 && stem_clocks(q1) * 1.3 >= c) ++q1;
-        const uint32_t end = l > 0 && q1 < k - 2 ? (uint32_t)(binom().c[q1][l] * d.ncl) : items;
+        const uint32_t end = l > 0 && q1 < k - 2 ? (uint32_t)(binom().c[q1][l] * ncl) : items;
         add(at, end, l > 0 ? fpk::kSplitGroups * std::max<uint64_t>(1, (uint64_t)(target / c)) : 1, 0, k - 2);
         at = std::max(at, end);
         q = q1;
@@ -927,12 +918,12 @@ void plan_split(Prepared *P, int ctas) {
       // a task of least size: one unit for each warpgroup, or one in all with its tails split
       const double unit_max = kStepClocks + tile * cut->blocks[0].tiles;
       const double target0 = std::max(kTaskClocks, std::min(total / C, 4 * kTaskClocks));
-      d.esplit = fpk::kSplitGroups * unit_max <= 1.5 * target0 ? 0 : 1;
-      const uint64_t parts = d.esplit ? 1 : fpk::kSplitGroups;
+      esplit = fpk::kSplitGroups * unit_max > 1.5 * target0;
+      const uint64_t parts = esplit ? 1 : fpk::kSplitGroups;
       double rem = total;
       for (uint32_t blk = 0; blk < cut->blocks.size(); ++blk) {
         const TailCut::Block &x = cut->blocks[blk];
-        const uint64_t ns = l > 0 ? binom().c[x.zhi][l] * d.ncl : 1;
+        const uint64_t ns = l > 0 ? binom().c[x.zhi][l] * ncl : 1;
         const uint32_t units = (uint32_t)((ns + 127) / 128);
         auto tiles_at = [&](int q) { return l > 0 && x.at >= 0 ? cut->tiles_at[x.at + q] : x.tiles; };
         // runs of units whose first stem meets about the same number of tiles
@@ -942,7 +933,7 @@ void plan_split(Prepared *P, int ctas) {
           int q1 = q + 1;
           while (l > 0 && q1 < x.zhi && tiles_at(q1) * 8 >= tiles * 7) ++q1;
           uint32_t end = units;
-          if (l > 0 && q1 < x.zhi) end = std::min<uint32_t>(units, (uint32_t)(binom().c[q1][l] * d.ncl / 128));
+          if (l > 0 && q1 < x.zhi) end = std::min<uint32_t>(units, (uint32_t)(binom().c[q1][l] * ncl / 128));
           if (end > at) {
             const double unit = kStepClocks + tile * tiles;
             const double target = std::max(kTaskClocks, rem / (2 * C));
@@ -955,6 +946,7 @@ void plan_split(Prepared *P, int ctas) {
         }
       }
     }
+    d.set_split(t, direct, esplit, nb, ncl);
     d.nseg = (uint32_t)P->split_segs.size() - d.seg_off;
     d.ntasks = tasks;
   }
@@ -1287,23 +1279,23 @@ template <int DB, class F>
 void split_walk(const fph::Prepared &P, const fpk::PassDesc &d, int pass, uint64_t lo, uint64_t hi, uint32_t block,
                 int zhi, F emit) {
   const fpenum::Binom &B = fph::binom();
-  const int k = P.k, b = P.p - 1, g = d.g, t = d.tail_rows, l = g - t;
-  const uint32_t etot = fpk::tails_above(B, k, t, b, -1), first = block * d.block;
-  const uint32_t nb = std::min(d.block, etot - first);
-  const uint32_t slices = d.esplit ? fpk::kSplitGroups : 1, parts = d.esplit ? 1 : fpk::kSplitGroups;
-  const uint64_t ns = l > 0 ? B(zhi, l) * d.ncl : 1;
-  const uint32_t lanes = d.direct ? 1 : fpk::kSplitGroup, tile = d.direct ? fpk::kSplitGroup : fpk::kSplitN;
+  const int k = P.k, b = P.p - 1, g = d.g, t = d.tail_rows(), l = g - t;
+  const uint32_t etot = fpk::tails_above(B, k, t, b, -1), first = block * d.block();
+  const uint32_t nb = std::min(d.block(), etot - first);
+  const uint32_t slices = d.esplit() ? fpk::kSplitGroups : 1, parts = d.esplit() ? 1 : fpk::kSplitGroups;
+  const uint64_t ns = l > 0 ? B(zhi, l) * d.ncl() : 1;
+  const uint32_t lanes = d.direct() ? 1 : fpk::kSplitGroup, tile = d.direct() ? fpk::kSplitGroup : fpk::kSplitN;
   const uint64_t share = (hi - lo + parts - 1) / parts;
   for (uint32_t grp = 0; grp < fpk::kSplitGroups; ++grp) {
-    const uint32_t part = d.esplit ? 0 : grp, slice = d.esplit ? grp : 0;
+    const uint32_t part = d.esplit() ? 0 : grp, slice = d.esplit() ? grp : 0;
     const uint64_t u0 = std::min(lo + part * share, hi), steps = std::min(u0 + share, hi) - u0, J0 = u0 * lanes;
     if (steps == 0 || J0 >= ns) continue;
-    const int q0 = l > 0 ? fpk::comb_floor(B, l - 1, k - t - 1, l, d.ncl, J0) : -1;
+    const int q0 = l > 0 ? fpk::comb_floor(B, l - 1, k - t - 1, l, d.ncl(), J0) : -1;
     const uint32_t tiles = (std::min(nb, fpk::tails_above(B, k, t, b, q0) - first) + tile - 1) / tile;
     for (uint32_t lane = 0; lane < lanes; ++lane) {
       const uint64_t J = J0 + lane * steps, nst = J < ns ? std::min(steps, ns - J) : 0;
       fpk::StemPos pf{-1, 0, 0};
-      if (nst && l > 0) pf = fpk::stem_unrank<DB>(B, J, k, t, l, b, d.ncl);
+      if (nst && l > 0) pf = fpk::stem_unrank<DB>(B, J, k, t, l, b, d.ncl());
       for (uint64_t i = 0; i < nst; ++i) {
         for (uint32_t c = slice; c < tiles; c += slices)
           for (uint32_t e = c * tile; e < std::min((c + 1) * tile, nb); ++e) {
@@ -1363,16 +1355,13 @@ int64_t fpcode_test_split_pass(fpcode_prepared *prep, int pass, int ctas, int ta
   }
   const int l = d.g - tail_rows;
   if (tail_rows < 2 || tail_rows > 3 || l < 0 || block < 1 || unit < 1 || esplit < 0 || esplit > 1) return -1;
-  d.direct = 0;
-  d.tail_rows = (uint8_t)tail_rows;
-  d.block = (uint32_t)block;
-  d.esplit = (uint8_t)esplit;
-  d.ncl = l > 0 ? (uint64_t)(b / 2) : 1;
-  for (int i = 1; i < l; ++i) d.ncl *= (uint64_t)b;
+  uint64_t ncl = l > 0 ? (uint64_t)(b / 2) : 1;
+  for (int i = 1; i < l; ++i) ncl *= (uint64_t)b;
+  d.set_split(tail_rows, false, esplit != 0, (uint32_t)block, ncl);
   const uint32_t etot = fpk::tails_above(fph::binom(), k, tail_rows, b, -1);
   for (uint32_t first = 0, blk = 0; first < etot; first += (uint32_t)block, ++blk) {
     const int zhi = fpk::tail_unrank(fph::binom(), first, k, tail_rows, b).z;
-    const uint64_t units = ((l > 0 ? fph::binom()(zhi, l) * d.ncl : 1) + 127) / 128;
+    const uint64_t units = ((l > 0 ? fph::binom()(zhi, l) * ncl : 1) + 127) / 128;
     for (uint64_t u = 0; u < units; u += (uint64_t)unit) walk(u, std::min<uint64_t>(u + unit, units), blk, zhi);
   }
   return n;

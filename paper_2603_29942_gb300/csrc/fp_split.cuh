@@ -9,7 +9,7 @@
 // Tails are numbered by z descending, so the tails with z > q come first:
 //   t = 2: z descending, x ascending, c_x ascending;
 //   t = 3: z descending, y descending, c_y ascending, x ascending, c_x.
-// They are cut into blocks of PassDesc.block entries, one block of which a
+// They are cut into blocks of PassDesc::block() entries, one block of which a
 // CTA holds in shared memory at a time.  Stems of a block are those with q
 // below the z of its first tail, numbered by q ascending, then by the
 // revolving-door rank of the other rows, then by the reflected Gray code of

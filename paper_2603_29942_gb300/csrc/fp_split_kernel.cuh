@@ -350,20 +350,20 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
   const Claim &cl = sh.task[buf].cl;
   constexpr int DB = P == 3 ? 1 : 4, RW = R * W, b = P - 1;
   constexpr unsigned FULL = 0xffffffffu;
-  const int k = sd.k, g = pd.g, t = pd.tail_rows, l = g - t;
+  const int k = sd.k, g = pd.g, t = pd.tail_rows(), l = g - t;
   const int lane = threadIdx.x & 31, row = threadIdx.x & (kSplitGroup - 1);
   const int warp = __shfl_sync(FULL, (int)(threadIdx.x >> 5), 0), grp = warp / (kSplitGroup / 32);
   const uint32_t mbar = smem_u32(&sh.product[grp]), near = smem_u32(&sh.near[buf]);
   const bool pair = sd.pair_sigp > 0;
-  const uint64_t ncl = pd.ncl;
+  const uint64_t ncl = pd.ncl();
   const uint32_t etot = tails_above(B, k, t, b, -1);
-  const uint32_t first = cl.block * pd.block, nb = min(pd.block, etot - first);
+  const uint32_t first = cl.block * pd.block(), nb = min(pd.block(), etot - first);
   const uint64_t ns = l > 0 ? B(cl.zhi, l) * ncl : 1ull;
-  const int K = sd.split_k, nu = sd.split_nu;
+  const int K = sd.split_k(), nu = sd.split_nu();
   uint32_t seen = 0;  // this lane's stem-tail pairs (a task's fit 32 bits): two codewords each, or one (l = 0)
   // the warpgroup's units [u0, u0 + steps) and its slice of the tails
-  const uint32_t parts = pd.esplit ? 1u : (uint32_t)kSplitGroups, part = pd.esplit ? 0u : (uint32_t)grp;
-  const uint32_t slices = pd.esplit ? (uint32_t)kSplitGroups : 1u, slice = pd.esplit ? (uint32_t)grp : 0u;
+  const uint32_t parts = pd.esplit() ? 1u : (uint32_t)kSplitGroups, part = pd.esplit() ? 0u : (uint32_t)grp;
+  const uint32_t slices = pd.esplit() ? (uint32_t)kSplitGroups : 1u, slice = pd.esplit() ? (uint32_t)grp : 0u;
   const uint32_t share = ((uint32_t)(cl.uhi - cl.ulo) + parts - 1) / parts;
   const uint64_t u0 = min(cl.ulo + (uint64_t)part * share, cl.uhi);
   const uint32_t steps = (uint32_t)(min(u0 + share, cl.uhi) - u0);
@@ -396,7 +396,7 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
   for (int q = 0; q < RW; ++q) x.s[q] = 0;
   x.pos = StemPos{-1, 0, 0};
 
-  if (pd.direct) {
+  if (pd.direct()) {
     // few codewords: one stem per warpgroup at a time, its tails over the 128
     // lanes, every weight exact (no table; before the first records most bounds would
     // pass the threshold anyway)
@@ -721,7 +721,7 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
               tk.stage = tk.build = tk.drop = 0;
               if (!tk.cl.skip) {
                 // a direct pass needs the packed tails only, which a built table of the same block has too
-                const int need = tk.pd.g < 2 ? 0 : tk.pd.direct ? 1 : 2, bt = tk.pd.tail_rows << 16 | (int)tk.pd.block;
+                const int need = tk.pd.g < 2 ? 0 : tk.pd.direct() ? 1 : 2, bt = tk.pd.tail_rows() << 16 | (int)tk.pd.block();
                 tk.stage = staged_j != tk.pd.j;
                 if (need && (tk.stage || built != bt || built_block != tk.cl.block || built_n < need)) {
                   tk.build = need;
@@ -778,7 +778,7 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
     const SlotDesc &sd = s_cc.sd;
     uint32_t *mult = reinterpret_cast<uint32_t *>(smem + kBinomBytes);
     uint32_t *tails = reinterpret_cast<uint32_t *>(smem + split_off_tails(sd.k, P, sd.rwpad));
-    char *table = smem + split_off_table(sd.k, P, sd.rwpad, sd.split_cap);
+    char *table = smem + split_off_table(sd.k, P, sd.rwpad, sd.split_cap());
     uint32_t parity = 0;
     for (uint32_t n = 0;; ++n) {
       const int b = (int)(n & 1u);
@@ -799,9 +799,9 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
           workers_sync();
         }
         if (tk.build && !tk.drop) {
-          const uint32_t etot = tails_above(binom, sd.k, tk.pd.tail_rows, P - 1, -1), first = tk.cl.block * tk.pd.block;
-          build_tails<P, R, W>(tails, table, mult, binom, sd.k, tk.pd.tail_rows, first, min(tk.pd.block, etot - first),
-                               sd.split_k, sd.split_nu, tk.build == 2);
+          const uint32_t etot = tails_above(binom, sd.k, tk.pd.tail_rows(), P - 1, -1), first = tk.cl.block * tk.pd.block();
+          build_tails<P, R, W>(tails, table, mult, binom, sd.k, tk.pd.tail_rows(), first, min(tk.pd.block(), etot - first),
+                               sd.split_k(), sd.split_nu(), tk.build == 2);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the tensor cores read the table
           workers_sync();
         }

@@ -58,13 +58,20 @@ struct PassDesc {
   uint32_t seg_off;        // pair-leaf passes: first segment of the pass in the code's segment list
   uint32_t nseg;           // pair-leaf passes: its segments (0: a one-row-leaf pass)
   uint32_t task_off;       // a slice of the pass (fpcode_prepared_pass_slice): its first task in the pass's plan
-  // Split passes (fp_split.cuh; then seg_off and nseg count SplitSegs).
-  uint64_t ncl;            // coefficient vectors per stem row subset
-  uint32_t block;          // tails per block
-  uint8_t tail_rows;       // rows of a tail (2 or 3)
-  uint8_t direct;          // 1: few codewords, every weight exact
-  uint8_t esplit;          // 1: a CTA's warpgroups share a task's stems and split its tails
-  uint8_t pad0;
+  // A split pass (fp_split.cuh) keeps its shape in four fields that only
+  // one-row plans use, so that the leaf kernels copy no more per pass:
+  // seg_off and nseg count SplitSegs then.
+  FPK_HD void set_split(int tail_rows, bool direct, bool esplit, uint32_t block, uint64_t ncl) {
+    pl = tail_rows | (direct ? 4 : 0) | (esplit ? 8 : 0);
+    unit = block;
+    phases = (uint32_t)ncl;
+    plan_ctas = (uint32_t)(ncl >> 32);
+  }
+  FPK_HD int tail_rows() const { return pl & 3; }           // rows of a tail (2 or 3)
+  FPK_HD bool direct() const { return (pl & 4) != 0; }      // few codewords: every weight exact
+  FPK_HD bool esplit() const { return (pl & 8) != 0; }      // a CTA's warpgroups share a task's stems and split its tails
+  FPK_HD uint32_t block() const { return unit; }            // tails per block
+  FPK_HD uint64_t ncl() const { return (uint64_t)plan_ctas << 32 | phases; }  // coefficient vectors per stem row subset
 };
 
 // Words per row of the pair-signature table (Mersenne p = 3, 7): for each
@@ -130,7 +137,7 @@ FPK_HD void task_range(const PassDesc &d, uint64_t t, uint64_t *lo, uint64_t *hi
   *lo = row0 * kThreads;
   *hi = (row0 + nrow) * kThreads < N ? (row0 + nrow) * kThreads : N;
 }
-static_assert(sizeof(PassDesc) == 96, "PassDesc layout");
+static_assert(sizeof(PassDesc) == 80, "PassDesc layout");
 
 // ---------------------------------------------------------------------------
 // Pair leaves (p = 3, 7).  A codeword of pass g >= 3 with rows T splits into
@@ -239,11 +246,15 @@ struct SlotDesc {
   const PassDesc *passes;        // npasses entries, device
   uint64_t seq;                  // serving: ticket of the code in this slot
   unsigned long long *pass_times;  // optional: %globaltimer at each pass end (device)
-  int32_t split_k, split_nu;     // split passes: class values per row (0: none), positions compared
-  int32_t split_cap;             // split passes: tails a CTA holds at a time
-  int32_t pad0;
+  // Tensor-core kernel (fp_split.cuh): class values per row, positions
+  // compared and tails held at a time, in the field of the pair bound that it
+  // does not use.
+  FPK_HD void set_split(int K, int nu, int cap) { pair_quick_max = K << 24 | nu << 16 | cap; }
+  FPK_HD int split_k() const { return (int)((uint32_t)pair_quick_max >> 24); }
+  FPK_HD int split_nu() const { return pair_quick_max >> 16 & 255; }
+  FPK_HD int split_cap() const { return pair_quick_max & 0xFFFF; }
 };
-static_assert(sizeof(SlotDesc) == 112, "SlotDesc layout");
+static_assert(sizeof(SlotDesc) == 96, "SlotDesc layout");
 
 // Dynamic state of one code, device memory (all zero = fresh).  Three
 // 128-byte lines keep apart what is written at different rates: the task
