@@ -91,6 +91,10 @@ int fpcode_test_pair_mode(const fpcode_prepared *prep, int pass, uint64_t J, uin
  * zeros), followed by slice 0 of B (W words).  `sig` holds up to 12 words.
  * Returns the number of words, or a negative status. */
 int fpcode_test_pair_entry(const fpcode_prepared *prep, int j, uint32_t e, uint32_t *sig);
+/* Class labels of 32 symbols of F_p (p = 5, 11 .. 251), the kernels' own
+ * code on the host: bit i of symbol q's label is bit q of label[i],
+ * i < r - 1.  Returns r - 1, or a negative status. */
+int fpcode_test_class_label(int p, const uint8_t *symbols, uint32_t *label);
 /* The pair table of Gamma_j as the kernels build it in shared memory
  * (Sec. 4.3 with pair leaves): one CTA stages the set's multiples, runs the
  * builder and copies the table out: all entries' pair_sigp signature words

@@ -194,6 +194,7 @@ def _declare(lib):
                                                 ctypes.POINTER(fpcode_opts)]),
         "fpcode_test_pair_mode": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_uint64, ctypes.POINTER(ctypes.c_uint32)]),
         "fpcode_test_key_coefficients": (ctypes.c_int, [_VP, ctypes.c_uint64, _IP, _IP, _IP]),
+        "fpcode_test_class_label": (ctypes.c_int, [ctypes.c_int, ctypes.c_char_p, ctypes.POINTER(ctypes.c_uint32)]),
         "fpcode_test_pair_entry": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_uint32, ctypes.POINTER(ctypes.c_uint32)]),
         "fpcode_test_lane_ranges": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                    ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64),
@@ -813,6 +814,16 @@ def fpcode_test_pair_mode(prep: Prepared, pass_index: int = -1, J: int = 0):
     if w < 0:
         raise FpcodeError(-w, "fpcode_test_pair_mode")
     return w if pass_index < 0 else (w, int(e.value))
+
+
+def fpcode_test_class_label(p: int, symbols) -> list[int]:
+    """Class labels of up to 32 symbols of F_p, one integer each."""
+    syms = [int(x) for x in symbols]
+    out = (ctypes.c_uint32 * 8)()
+    n = lib().fpcode_test_class_label(int(p), bytes(syms + [0] * (32 - len(syms))), out)
+    if n < 0:
+        raise FpcodeError(-n, "fpcode_test_class_label")
+    return [sum(((out[i] >> q) & 1) << i for i in range(n)) for q in range(len(syms))]
 
 
 def fpcode_test_pair_entry(prep: Prepared, j: int, e: int) -> list[int]:

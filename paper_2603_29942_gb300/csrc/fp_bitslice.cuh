@@ -197,6 +197,35 @@ FP_HD void neg_mersenne(const uint32_t *a, uint32_t *s) {
   for (int i = 0; i < R; ++i) s[i] = ~a[i] & m;
 }
 
+// Class label of {v, -v}: R - 1 slices, the same for v and p - v and for no
+// other symbol, 0 only for 0.  So S + y and S - y are both nonzero exactly
+// where the labels of S and y differ, and one comparison of R - 1 slices
+// stands for two isometric subtractions.  p = 2^R - 1: neighbouring slices
+// differ alike in v and its complement.  p = 5: {1,4} = 01, {2,3} = 10.
+// Else: one of v and p - v is even (p is odd); the label is half of that
+// one, v >> 1 or (p-1)/2 - (v >> 1) = ~(v >> 1) + (p+1)/2.
+template <int P, int R>
+FP_HD void class_label(const uint32_t *s, uint32_t *a, int p) {
+  if (P == 5) {
+    a[0] = s[1];
+    a[1] = s[2] | (s[0] & ~s[1]);
+  } else if (P == (1 << R) - 1) {
+#pragma unroll
+    for (int i = 0; i + 1 < R; ++i) a[i] = s[i] ^ s[i + 1];
+  } else {
+    const int h1 = (p + 1) / 2;
+    const uint32_t odd = s[0];
+    uint32_t c = 0;
+#pragma unroll
+    for (int i = 0; i + 1 < R; ++i) {
+      const uint32_t x = s[i + 1] ^ odd;
+      const uint32_t k = ((h1 >> i) & 1) ? odd : 0u;
+      a[i] = x ^ k ^ c;
+      c = (x & k) | (x & c) | (k & c);
+    }
+  }
+}
+
 // Multiplication by 2^t for p = 2^r - 1: circular shift of the slice index
 // (Sec. 4.2: 3 * 2 = (0,1,1), 3 * 4 = (1,0,1) in F_7).
 template <int R>

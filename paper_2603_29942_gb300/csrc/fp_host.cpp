@@ -313,7 +313,7 @@ int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prep
     mix(tail);
     P->code_hash = h;
   }
-  if (P->smem_bytes_per_set() > 96 * 1024) {
+  if (P->smem_bytes_per_set() > (size_t)fpk::kSetBytesMax) {
     set_error("bit-sliced multiples of one information set exceed 96 KiB (k (p-1) r W too large)");
     return FPCODE_EINVAL;
   }
@@ -1399,6 +1399,25 @@ int fpcode_test_prepared_row(const fpcode_prepared *prep, int j, int t, int v, u
     std::memcpy(sig, sg, (size_t)SIG * sizeof(uint32_t));
   }
   return SIG;
+}
+
+int fpcode_test_class_label(int p, const uint8_t *symbols, uint32_t *label) {
+  if (!symbols || !label || p < 5 || p == 7 || p > 251 || !(p & 1)) return -FPCODE_EINVAL;
+  const int r = fpbs::bits_for(p);
+  uint32_t s[8] = {0};
+  for (int q = 0; q < 32; ++q) {
+    if (symbols[q] >= p) return -FPCODE_EINVAL;
+    for (int i = 0; i < r; ++i) s[i] |= (uint32_t)((symbols[q] >> i) & 1) << q;
+  }
+  if (p == 5) fpbs::class_label<5, 3>(s, label, p);
+  else if (p == 31) fpbs::class_label<31, 5>(s, label, p);
+  else if (p == 127) fpbs::class_label<127, 7>(s, label, p);
+  else if (r == 4) fpbs::class_label<0, 4>(s, label, p);
+  else if (r == 5) fpbs::class_label<0, 5>(s, label, p);
+  else if (r == 6) fpbs::class_label<0, 6>(s, label, p);
+  else if (r == 7) fpbs::class_label<0, 7>(s, label, p);
+  else fpbs::class_label<0, 8>(s, label, p);
+  return r - 1;
 }
 
 int fpcode_test_pair_entry(const fpcode_prepared *prep, int j, uint32_t e, uint32_t *sig) {

@@ -73,8 +73,8 @@ struct Prepared {
                 : (size_t)k * ((size_t)(p - 1) * rwpad + fpk::sig_words(p, r, W));
   }
   size_t table_bytes_per_set() const { return table_words_per_set() * 4; }
-  // Shared memory one staged information set takes (with the pair table).
-  size_t smem_bytes_per_set() const { return (table_words_per_set() + pair_words_per_set()) * 4; }
+  // Shared memory one staged information set takes (with the pair table or the class labels).
+  size_t smem_bytes_per_set() const { return (table_words_per_set() + pair_words_per_set() + (size_t)fpk::set_label_words(p, r, W, k)) * 4; }
 };
 
 // Guided share of a pair-leaf pass (task_share, or its default for a pass

@@ -249,23 +249,34 @@ __device__ void task_rows(const SlotDesc &sd, int pass, const uint32_t *tab, int
 // S + y = 0 iff d is all ones and S - y = 0 iff d is all zeros (negation is
 // the bitwise complement), so that mask is OR_i (d_i xor d_{i+1}) =
 // OR_i ((S_i xor S_{i+1}) xor (y_i xor y_{i+1})): the prefix keeps its r-1
-// "signature" words, the row table stores the leaf's.  Other primes AND the
-// two isometric subtractions.  One POPC per word covers two codewords (for
-// p = 3 both leaf coefficients); only a pair whose bound is below the
-// current threshold is evaluated exactly (slow path).
+// "signature" words, the row table stores the leaf's.  Other primes compare
+// class labels of r-1 slices in the same way (fpbs::class_label; p = 5 both
+// labels of a row in one entry, else one entry per multiple).  One POPC per
+// word covers two codewords (for p = 3 both leaf coefficients); only a pair
+// whose bound is below the current threshold is evaluated exactly (slow
+// path).  Sets whose labels do not fit in shared memory AND the two
+// isometric subtractions: 2 R W words read and 2 R W LOP3s a pair instead of
+// (R - 1) W of each.  The loop is bound by those shared-memory reads (16
+// bytes to each of 32 lanes take 4 cycles of an SM): F_31 [70,10], 8.6e8
+// codewords, 1017 us with the subtractions, 576 us with labels.
 // ---------------------------------------------------------------------------
 template <int P, int R, int W>
 struct LeafFilter {
-  static constexpr bool kMersenne = (P == 3 || P == 7);
-  static constexpr int kSigW = kMersenne ? (((P == 3 ? W * (R - 1) : 3 * W * (R - 1)) + 3) & ~3) : 0;
-  static constexpr int kPrefSig = kMersenne ? W * (R - 1) : 1;
+  static constexpr bool kRowSig = P == 3 || P == 5 || P == 7;  // a row's signatures are one entry
+  static constexpr bool kLabels = !kRowSig && label_shape(R, W);  // one entry per multiple, where a set's fit
+  static constexpr int kSigW = kRowSig ? ((P - 1) / 2 * W * (R - 1) + 3) & ~3 : (W * (R - 1) + 3) & ~3;
+  static constexpr int kPrefSig = kRowSig || kLabels ? W * (R - 1) : 1;
   // leaves evaluated per vote: as many as the registers allow
-  static constexpr int kUnroll = !kMersenne ? 1 : kSigW <= 4 ? 4 : kSigW <= 8 ? 2 : 1;
+  static constexpr int kUnroll = !kRowSig ? 1 : kSigW <= 4 ? 4 : kSigW <= 8 ? 2 : 1;
   // The one-popcount bound of W > 1 words (popc of the words' OR) is used
   // while the threshold is at most this: about 32 (1 - q^W) - 8, eight
   // under the bound's mean for random symbols, where q is the chance that
-  // a position is zero in a word's pair mask (5/9 for p = 3, 13/49 for p = 7).
-  static constexpr int kQuickMax = P == 3 ? (W == 2 ? 14 : W == 3 ? 18 : 21) : P == 7 ? (W == 2 ? 21 : 23) : 0;
+  // a position is zero in a word's pair mask (5/9 for p = 3, 9/25 for p = 5,
+  // 13/49 for p = 7).
+  static constexpr int kQuickMax = P == 3   ? (W == 2 ? 14 : W == 3 ? 18 : 21)
+                                   : P == 5 ? (W == 2 ? 19 : W == 3 ? 22 : 23)
+                                   : P == 7 ? (W == 2 ? 21 : 23)
+                                            : 0;
 };
 
 // Lower bound on the redundant weight of S + c A[x] over every nonzero
@@ -275,13 +286,14 @@ struct BoolTag {
   static constexpr bool value = B;
 };
 
+// QUICK: row signatures, the one-popcount bound; other primes: labels.
 template <int P, int R, int W, bool QUICK, int NA>
 __device__ __forceinline__ int pair_bound(const uint32_t (&s)[R * W], const uint32_t (&a)[NA], const uint32_t *sig,
                                           const uint32_t *tab, int x, int p) {
   using F = LeafFilter<P, R, W>;
   constexpr int RWP = Shape<R, W>::RWP;
   int best = 1 << 20;
-  if constexpr (F::kMersenne) {
+  if constexpr (F::kRowSig) {
     uint32_t e[F::kSigW];
     load_entry<F::kSigW>(sig, x, e);
     constexpr int NP = (P - 1) / 2;
@@ -308,6 +320,22 @@ __device__ __forceinline__ int pair_bound(const uint32_t (&s)[R * W], const uint
         }
         best = min(best, lb);
       }
+    }
+  } else if constexpr (F::kLabels && QUICK) {
+    const int np = (p - 1) / 2;
+#pragma unroll 3
+    for (int q = 0; q < np; ++q) {
+      uint32_t e[F::kSigW];
+      load_entry<F::kSigW>(sig, x * np + q, e);
+      int lb = 0;
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        uint32_t f = 0;
+#pragma unroll
+        for (int i = 0; i + 1 < R; ++i) f |= a[w * (R - 1) + i] ^ e[w * (R - 1) + i];
+        lb += __popc(f);
+      }
+      best = min(best, lb);
     }
   } else {
     const int b = p - 1;
@@ -344,13 +372,18 @@ __device__ __forceinline__ void leaf_exact(const uint32_t (&s)[R * W], const uin
   }
 }
 
-template <int R, int W, int NA>
-__device__ __forceinline__ void prefix_signature(const uint32_t (&s)[R * W], uint32_t (&a)[NA]) {
+template <int P, int R, int W, int NA>
+__device__ __forceinline__ void prefix_signature(const uint32_t (&s)[R * W], uint32_t (&a)[NA], int p) {
   static_assert(NA >= W * (R - 1), "signature size");
 #pragma unroll
-  for (int w = 0; w < W; ++w)
+  for (int w = 0; w < W; ++w) {
+    if constexpr (P == 3 || P == 7) {
 #pragma unroll
-    for (int i = 0; i + 1 < R; ++i) a[w * (R - 1) + i] = s[w * R + i] ^ s[w * R + i + 1];
+      for (int i = 0; i + 1 < R; ++i) a[w * (R - 1) + i] = s[w * R + i] ^ s[w * R + i + 1];
+    } else {
+      fpbs::class_label<P, R>(&s[w * R], &a[w * (R - 1)], p);
+    }
+  }
 }
 
 template <int P, int R, int W, int DB, int UNR>
@@ -365,7 +398,8 @@ __device__ void task_prefixes(const SlotDesc &sd, const PassDesc &pd, int pass, 
   const int k = sd.k;
   const int g = pd.g;
   const int L = g - 2;
-  const uint32_t *sig = tab + k * b * RWP;  // pair signatures (Mersenne p)
+  const uint32_t *sig = tab + k * b * RWP;  // pair signatures or class labels
+  const bool labels = F::kLabels && set_label_words(p, R, W, k) > 0;
   const uint64_t pu = (uhi - ulo + kThreads - 1) / kThreads;  // units per lane, same for the CTA
   const uint64_t unit = pd.unit;
   const uint64_t pl = pu * unit;                               // prefix steps
@@ -390,7 +424,7 @@ __device__ void task_prefixes(const SlotDesc &sd, const PassDesc &pd, int pass, 
     ci = (I - fpenum::prefixes_below(B, pf.m, g, pd.NC)) - pf.qi * pd.NC;
     nq = B(pf.m, L);
     build_sum<P, R, W, DB>(s, tab, pf, L, b, p, qrows);
-    if constexpr (F::kMersenne) prefix_signature<R, W>(s, a);
+    if constexpr (F::kRowSig || F::kLabels) prefix_signature<P, R, W>(s, a, p);
   }
 
   // prefixes left to this lane (the current one included); its index is Iend - left
@@ -468,6 +502,9 @@ __device__ void task_prefixes(const SlotDesc &sd, const PassDesc &pd, int pass, 
     if constexpr (W > 1 && UNR > 1) {  // single-code kernels; the batched ones keep one copy
       if (thr <= F::kQuickMax) leaves(BoolTag<true>{});  // thr is the same on every lane here
       else leaves(BoolTag<false>{});
+    } else if constexpr (F::kLabels) {
+      if (labels) leaves(BoolTag<true>{});
+      else leaves(BoolTag<false>{});
     } else {
       leaves(BoolTag<false>{});
     }
@@ -483,7 +520,7 @@ __device__ void task_prefixes(const SlotDesc &sd, const PassDesc &pd, int pass, 
         build_sum<P, R, W, DB>(s, tab, pf, L, b, p, qrows);
         cw = (uint32_t)(k - 1 - pf.m) * (uint32_t)b;
       }
-      if constexpr (F::kMersenne) prefix_signature<R, W>(s, a);
+      if constexpr (F::kRowSig || F::kLabels) prefix_signature<P, R, W>(s, a, p);
     }
     left -= left > 0 ? 1u : 0u;
    }
@@ -539,6 +576,27 @@ __device__ __noinline__ void build_pairs(uint32_t *tab, int k, int rwpad, int si
       p0[e * W + w] = sum[0];
     }
     for (int q = W * (R - 1); q < sigp; ++q) pt[e * sigp + q] = 0u;
+  }
+}
+
+// Class labels of the staged information set, built by the CTA behind the
+// multiples: entry (row, q) for the multiple q + 1 of the row, label_words
+// each (zero-padded), word-major as in the sum's label.  One pass over the
+// multiples per staged set; built here they cost no upload.
+template <int P, int R, int W>
+__device__ __noinline__ void build_labels(uint32_t *tab, int k, int p) {
+  constexpr int RWP = Shape<R, W>::RWP;
+  constexpr int LS = P == 5 ? W * (R - 1) : (W * (R - 1) + 3) & ~3;
+  const int np = (p - 1) / 2;
+  uint32_t *lab = tab + k * (p - 1) * RWP;
+  for (int i = threadIdx.x; i < k * np; i += kThreads) {
+    const int t = i / np, q = i - t * np;
+    const uint32_t *e = tab + (t * (p - 1) + q) * RWP;
+    uint32_t *o = lab + i * LS;
+#pragma unroll
+    for (int w = 0; w < W; ++w) fpbs::class_label<P, R>(e + w * R, o + w * (R - 1), p);
+#pragma unroll
+    for (int z = W * (R - 1); z < LS; ++z) o[z] = 0u;
   }
 }
 
@@ -698,7 +756,7 @@ __device__ void task_pairs(const SlotDesc &sd, const PassDesc &pd, int pass, con
   uint32_t since = 0;
   for (uint32_t it = 0; it < nmax; ++it) {
     const bool act = it < nstem;
-    if constexpr (SW > 0) prefix_signature<R, W>(s, a);
+    if constexpr (SW > 0) prefix_signature<P, R, W>(s, a, P);
     const uint32_t E = act ? pair_entries_above(k, pf.m, b) : 0u;  // pf.m = -1 for g = 2
     const uint32_t nch = E / EPL;  // E is a multiple of EPL: even for p = 3, a multiple of 6 for p = 7
     const uint32_t its = nch > (uint32_t)sub ? ((nch - (uint32_t)sub + (1u << lsplit) - 1) >> lsplit) : 0u;
@@ -854,11 +912,24 @@ struct Fixed {
   static constexpr int DB = P == 3 ? 1 : (P == 5 || P == 7) ? 4 : 8;  // as the host's digit width
   static constexpr int kSegCache = PAIRS ? 768 : 1;  // pair-leaf segments held in shared memory
   static constexpr int kPassCache = 24;                // pass descriptors held in shared memory (one code)
-  // after staging a set: its pair table (pair-leaf codes), built in shared memory
-  static __device__ __forceinline__ void stage_pairs(uint32_t *tab, const SlotDesc &sd) {
-    if constexpr (PAIRS && (P == 3 || P == 7)) {
-      if (sd.pair_sigp > 0) build_pairs<P, R, W>(tab, sd.k, sd.rwpad, sd.pair_sigp);
+  // after staging a set: its pair table (pair-leaf codes) or its class
+  // labels, built in shared memory; false if it has neither
+  static __device__ __forceinline__ bool stage_derived(uint32_t *tab, const SlotDesc &sd) {
+    if constexpr (P == 3 || P == 7) {
+      if constexpr (PAIRS) {
+        if (sd.pair_sigp > 0) {
+          build_pairs<P, R, W>(tab, sd.k, sd.rwpad, sd.pair_sigp);
+          return true;
+        }
+      }
+    } else if constexpr (label_shape(R, W)) {
+      const int p = P ? P : sd.p;
+      if (set_label_words(p, R, W, sd.k) > 0) {
+        build_labels<P, R, W>(tab, sd.k, p);
+        return true;
+      }
     }
+    return false;
   }
   static __device__ __forceinline__ void run(const SlotDesc &sd, const PassDesc &pd, int pass, const uint32_t *tab,
                                              const fpenum::BinomCols &B, uint64_t ulo, uint64_t uhi, int lsplit,
@@ -887,7 +958,17 @@ template <int WMAX>
 struct Multi357 {
   static constexpr int kSegCache = 1;  // batches take one-row leaves
   static constexpr int kPassCache = 1;  // and read their pass descriptors from global memory
-  static __device__ __forceinline__ void stage_pairs(uint32_t *, const SlotDesc &) {}  // one-row leaves only
+  static __device__ __forceinline__ bool stage_derived(uint32_t *tab, const SlotDesc &sd) {  // one-row leaves only
+    if (sd.p != 5) return false;
+    switch (sd.W) {
+      case 1: build_labels<5, 3, 1>(tab, sd.k, 5); break;
+      case 2: build_labels<5, 3, 2>(tab, sd.k, 5); break;
+      case 3: if constexpr (WMAX >= 3) build_labels<5, 3, 3>(tab, sd.k, 5); break;
+      case 4: if constexpr (WMAX >= 4) build_labels<5, 3, 4>(tab, sd.k, 5); break;
+      default: break;
+    }
+    return true;
+  }
   static __device__ __forceinline__ void run(const SlotDesc &sd, const PassDesc &pd, int pass, const uint32_t *tab,
                                              const fpenum::BinomCols &B, uint64_t ulo, uint64_t uhi, int lsplit,
                                              int U, SlotState *st, SlotAux *ax, unsigned long long &count) {
@@ -1582,10 +1663,7 @@ __global__ void __launch_bounds__(kThreads, FPK_MIN_BLOCKS) bz_kernel(const Slot
           if (i0 + u * kThreads < nv) tab4[i0 + u * kThreads] = v[u];
       }
       __syncthreads();
-      if (s_cc.sd.pair_sigp > 0) {
-        V::stage_pairs(tab, s_cc.sd);
-        __syncthreads();
-      }
+      if (V::stage_derived(tab, s_cc.sd)) __syncthreads();  // the same answer on every thread
     }
     unsigned long long count = 0;
     SlotAux *ax = cs.aux + slot;

@@ -83,6 +83,26 @@ FPK_HD int sig_words(int p, int r, int W) {
 }
 FPK_HD int pair_rep(int p, int q) { return p == 7 ? (1 << q) : q + 1; }
 
+// Class labels (one-row leaves of the other primes): y and -y have the same
+// label of r - 1 bits (fpbs::class_label), so S + y and S - y are both
+// nonzero exactly where the labels of S and y differ.  The kernel puts the
+// labels of the multiples 1 .. (p-1)/2 of every row behind the staged
+// multiples of an information set.  Words of one multiple's label: whole
+// 16-byte vectors but for p = 5, whose two labels of a row are one entry.
+constexpr int kSetBytesMax = 96 * 1024;  // shared memory of one information set
+FPK_HD int label_words(int p, int r, int W) { return p == 5 ? W * (r - 1) : (W * (r - 1) + 3) & ~3; }
+// Labels are kept while a lane's sum and its label leave room in 64
+// registers (beyond: spills), and while they fit behind the multiples.
+FPK_HD constexpr bool label_shape(int r, int W) { return W * (2 * r - 1) <= 36; }
+// Words of an information set's labels; 0: none (p = 3 and 7 have row
+// signatures, and sets that would not fit take the two subtractions).
+FPK_HD int set_label_words(int p, int r, int W, int k) {
+  if (p == 3 || p == 7 || !label_shape(r, W)) return 0;
+  const int words = k * ((p - 1) / 2) * label_words(p, r, W);
+  const int rows = k * (p - 1) * ((r * W + 3) & ~3);
+  return (rows + words) * 4 <= kSetBytesMax ? words : 0;
+}
+
 // Variant id: prime class * 4 + (W - 1); classes 0: p = 3, 1: p = 5,
 // 2: p = 7, 3 + (r - 4): other primes with r bits (r = 4..8), 8: p = 31,
 // 9: p = 127 (the Mersenne primes above 7, with their own exact add).
