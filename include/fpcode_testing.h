@@ -95,6 +95,10 @@ int fpcode_test_pair_entry(const fpcode_prepared *prep, int j, uint32_t e, uint3
  * code on the host: bit i of symbol q's label is bit q of label[i],
  * i < r - 1.  Returns r - 1, or a negative status. */
 int fpcode_test_class_label(int p, const uint8_t *symbols, uint32_t *label);
+/* Logarithms of the classes {v, -v} of 32 symbols (p = 31, 127), and
+ * log s - log t of symbols s and t as the kernels take it: bit i of symbol
+ * q is bit q of word i, i < r - 1.  Returns r - 1, or a negative status. */
+int fpcode_test_class_log(int p, const uint8_t *s, const uint8_t *t, uint32_t *log_s, uint32_t *difference);
 /* The pair table of Gamma_j as the kernels build it in shared memory
  * (Sec. 4.3 with pair leaves): one CTA stages the set's multiples, runs the
  * builder and copies the table out: all entries' pair_sigp signature words

@@ -195,6 +195,8 @@ def _declare(lib):
         "fpcode_test_pair_mode": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_uint64, ctypes.POINTER(ctypes.c_uint32)]),
         "fpcode_test_key_coefficients": (ctypes.c_int, [_VP, ctypes.c_uint64, _IP, _IP, _IP]),
         "fpcode_test_class_label": (ctypes.c_int, [ctypes.c_int, ctypes.c_char_p, ctypes.POINTER(ctypes.c_uint32)]),
+        "fpcode_test_class_log": (ctypes.c_int, [ctypes.c_int, ctypes.c_char_p, ctypes.c_char_p,
+                                                 ctypes.POINTER(ctypes.c_uint32), ctypes.POINTER(ctypes.c_uint32)]),
         "fpcode_test_pair_entry": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_uint32, ctypes.POINTER(ctypes.c_uint32)]),
         "fpcode_test_lane_ranges": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                    ctypes.POINTER(ctypes.c_uint64), ctypes.POINTER(ctypes.c_uint64),
@@ -824,6 +826,16 @@ def fpcode_test_class_label(p: int, symbols) -> list[int]:
     if n < 0:
         raise FpcodeError(-n, "fpcode_test_class_label")
     return [sum(((out[i] >> q) & 1) << i for i in range(n)) for q in range(len(syms))]
+
+
+def fpcode_test_class_log(p: int, s, t) -> tuple[list[int], list[int]]:
+    """(log s, log s - log t) of up to 32 pairs of symbols, p = 31 or 127."""
+    s, t = [int(x) for x in s], [int(x) for x in t]
+    a, d = (ctypes.c_uint32 * 8)(), (ctypes.c_uint32 * 8)()
+    n = lib().fpcode_test_class_log(int(p), bytes(s + [0] * (32 - len(s))), bytes(t + [0] * (32 - len(t))), a, d)
+    if n < 0:
+        raise FpcodeError(-n, "fpcode_test_class_log")
+    return tuple([sum(((w[i] >> q) & 1) << i for i in range(n)) for q in range(len(s))] for w in (a, d))
 
 
 def fpcode_test_pair_entry(prep: Prepared, j: int, e: int) -> list[int]:

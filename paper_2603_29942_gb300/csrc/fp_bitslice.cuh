@@ -226,6 +226,69 @@ FP_HD void class_label(const uint32_t *s, uint32_t *a, int p) {
   }
 }
 
+// Any boolean function of N bit-slices: bit (a[N-1] .. a[0]) of the table.
+template <uint64_t TT, int N>
+FP_HD uint32_t lookup(const uint32_t *a) {
+  if constexpr (N == 0) {
+    return (TT & 1) ? 0xFFFFFFFFu : 0u;
+  } else {
+#ifdef __CUDA_ARCH__
+    if constexpr (N == 3) {
+      uint32_t f;
+      asm("lop3.b32 %0, %1, %2, %3, %4;" : "=r"(f) : "r"(a[2]), "r"(a[1]), "r"(a[0]), "n"((int)(TT & 0xFF)));
+      return f;
+    }
+#endif
+    constexpr int H = 1 << (N - 1);
+    constexpr uint64_t M = (1ull << H) - 1;
+    const uint32_t hi = lookup<((TT >> H) & M), N - 1>(a), lo = lookup<(TT & M), N - 1>(a);
+    return (hi & a[N - 1]) | (lo & ~a[N - 1]);
+  }
+}
+
+// Discrete logarithms of the classes {v, -v}, p = 2^R - 1 with primitive
+// root 3 (p = 31, 127): there are (p-1)/2 = 2^(R-1) - 1 classes, and class
+// 3^e has the logarithm e mod that number, R - 1 bits.  table(i): bit i of
+// the logarithm as a function of the class label.
+template <int P, int R>
+struct ClassLog {
+  static_assert(P == (1 << R) - 1 && (P == 31 || P == 127), "3 is a primitive root");
+  static constexpr uint64_t table(int bit) {
+    uint64_t t = 0;
+    int v = 1;
+    for (int e = 0; e < (P - 1) / 2; ++e, v = v * 3 % P)
+      if ((e >> bit) & 1) t |= 1ull << ((v ^ (v >> 1)) & (P >> 1));
+    return t;
+  }
+};
+template <int P, int R, int I = 0>
+FP_HD void class_log(const uint32_t *label, uint32_t *l) {
+  if constexpr (I < R - 1) {
+    l[I] = lookup<ClassLog<P, R>::table(I), R - 1>(label);
+    class_log<P, R, I + 1>(label, l);
+  }
+}
+
+// l + l' modulo 2^M - 1 in M slices, zero as all zeros or all ones (the
+// end-around carry cannot carry again: the sum without it is then at most
+// 2^M - 2 of 2^M).
+template <int M>
+FP_HD void add_logs(const uint32_t *a, const uint32_t *b, uint32_t *d) {
+  uint32_t c = 0;
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const uint32_t t = a[i] ^ b[i];
+    d[i] = t ^ c;
+    c = (a[i] & b[i]) | (t & c);
+  }
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    const uint32_t t = d[i] & c;
+    d[i] ^= c;
+    c = t;
+  }
+}
+
 // Multiplication by 2^t for p = 2^r - 1: circular shift of the slice index
 // (Sec. 4.2: 3 * 2 = (0,1,1), 3 * 4 = (1,0,1) in F_7).
 template <int R>

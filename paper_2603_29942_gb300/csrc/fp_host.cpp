@@ -1420,6 +1420,20 @@ int fpcode_test_class_label(int p, const uint8_t *symbols, uint32_t *label) {
   return r - 1;
 }
 
+int fpcode_test_class_log(int p, const uint8_t *s, const uint8_t *t, uint32_t *log_s, uint32_t *difference) {
+  uint32_t ls[8], lt[8], a[8], b[8];
+  if (!log_s || !difference || (p != 31 && p != 127) || fpcode_test_class_label(p, s, ls) < 0 ||
+      fpcode_test_class_label(p, t, lt) < 0)
+    return -FPCODE_EINVAL;
+  const int M = p == 31 ? 4 : 6;
+  if (M == 4) fpbs::class_log<31, 5>(ls, a), fpbs::class_log<31, 5>(lt, b);
+  else fpbs::class_log<127, 7>(ls, a), fpbs::class_log<127, 7>(lt, b);
+  for (int i = 0; i < M; ++i) log_s[i] = a[i], b[i] = ~b[i];
+  if (M == 4) fpbs::add_logs<4>(a, b, difference);
+  else fpbs::add_logs<6>(a, b, difference);
+  return M;
+}
+
 int fpcode_test_pair_entry(const fpcode_prepared *prep, int j, uint32_t e, uint32_t *sig) {
   const fph::Prepared *P = prep ? &prep->host : nullptr;
   if (!P || !P->pair || j < 0 || j >= P->m || !sig) return -FPCODE_EINVAL;

@@ -254,7 +254,20 @@ __device__ void task_rows(const SlotDesc &sd, int pass, const uint32_t *tab, int
 // labels of a row in one entry, else one entry per multiple).  One POPC per
 // word covers two codewords (for p = 3 both leaf coefficients); only a pair
 // whose bound is below the current threshold is evaluated exactly (slow
-// path).  Sets whose labels do not fit in shared memory AND the two
+// path).
+//
+// p = 31 and 127, up to 64 redundant positions: the logarithm of a class.
+// S + y = 0 or S - y = 0 for y = 3^e A[x] where log S - log A[x] = e modulo
+// the number of classes, 2^(R-1) - 1, so one end-around-carry subtraction of
+// R - 1 slices gives the class of every position for all multiples of the
+// row at once.  The mask of class e is then one AND of two products of
+// slices, and the row's bound is its most frequent class (plus positions
+// where both are zero).  One entry a row is read instead of (p-1)/2.  F_31
+// [70,10]: 576 us with one entry a multiple, 518 us so; F_127 [20,6] 127 and
+// 76 us (kernel).  The ALU pipe is 74 % busy, half of it with the steps from
+// one prefix to the next (2.5 leaf rows a prefix there).
+//
+// Sets whose labels do not fit in shared memory AND the two
 // isometric subtractions: 2 R W words read and 2 R W LOP3s a pair instead of
 // (R - 1) W of each.  The loop is bound by those shared-memory reads (16
 // bytes to each of 32 lanes take 4 cycles of an SM): F_31 [70,10], 8.6e8
@@ -265,7 +278,8 @@ struct LeafFilter {
   static constexpr bool kRowSig = P == 3 || P == 5 || P == 7;  // a row's signatures are one entry
   static constexpr bool kLabels = !kRowSig && label_shape(R, W);  // one entry per multiple, where a set's fit
   static constexpr int kSigW = kRowSig ? ((P - 1) / 2 * W * (R - 1) + 3) & ~3 : (W * (R - 1) + 3) & ~3;
-  static constexpr int kPrefSig = kRowSig || kLabels ? W * (R - 1) : 1;
+  static constexpr bool kLogs = log_labels(P, W);  // labels as logarithms, one entry per row
+  static constexpr int kPrefSig = kLogs ? W * R : kRowSig || kLabels ? W * (R - 1) : 1;
   // leaves evaluated per vote: as many as the registers allow
   static constexpr int kUnroll = !kRowSig ? 1 : kSigW <= 4 ? 4 : kSigW <= 8 ? 2 : 1;
   // The one-popcount bound of W > 1 words (popc of the words' OR) is used
@@ -321,6 +335,50 @@ __device__ __forceinline__ int pair_bound(const uint32_t (&s)[R * W], const uint
         best = min(best, lb);
       }
     }
+  } else if constexpr (F::kLogs && QUICK) {
+    constexpr int M = R - 1, N = 1 << (M / 2);
+    uint32_t e[RWP];
+    load_entry<RWP>(sig, x, e);
+    uint32_t lo[W][N], up[W][M / 2], nz[W];  // products of the lower slices; the upper slices
+    int both = 0;  // positions where S and A[x] are both zero (the padding too)
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      uint32_t d[M];
+      fpbs::add_logs<M>(&a[w * R], &e[w * R], d);
+      nz[w] = a[w * R + M] & e[w * R + M];
+      both += __popc(~(a[w * R + M] | e[w * R + M]));
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        lo[w][i] = 0xFFFFFFFFu;
+#pragma unroll
+        for (int q = 0; q < M / 2; ++q) lo[w][i] &= (i >> q) & 1 ? d[q] : ~d[q];
+      }
+#pragma unroll
+      for (int q = 0; q < M / 2; ++q) up[w][q] = d[M / 2 + q];
+    }
+    auto hi = [&](int w, int i) {
+      uint32_t h = nz[w];
+#pragma unroll
+      for (int q = 0; q < M / 2; ++q) h &= (i >> q) & 1 ? up[w][q] : ~up[w][q];
+      return h;
+    };
+    int most = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      uint32_t h[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w) h[w] = hi(w, i);
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        if (i == N - 1 && j == N - 1) continue;  // all ones: class 0 again
+        int z = 0;
+#pragma unroll
+        for (int w = 0; w < W; ++w)
+          z += __popc(i == 0 && j == 0 ? (h[w] & lo[w][0]) | (hi(w, N - 1) & lo[w][N - 1]) : h[w] & lo[w][j]);
+        most = max(most, z);
+      }
+    }
+    best = 32 * W - both - most;
   } else if constexpr (F::kLabels && QUICK) {
     const int np = (p - 1) / 2;
 #pragma unroll 3
@@ -380,6 +438,11 @@ __device__ __forceinline__ void prefix_signature(const uint32_t (&s)[R * W], uin
     if constexpr (P == 3 || P == 7) {
 #pragma unroll
       for (int i = 0; i + 1 < R; ++i) a[w * (R - 1) + i] = s[w * R + i] ^ s[w * R + i + 1];
+    } else if constexpr (log_labels(P, W)) {
+      uint32_t lab[R - 1];
+      fpbs::class_label<P, R>(&s[w * R], lab, p);
+      fpbs::class_log<P, R>(lab, &a[w * R]);
+      a[w * R + R - 1] = fpbs::nz<R>(&s[w * R]);
     } else {
       fpbs::class_label<P, R>(&s[w * R], &a[w * (R - 1)], p);
     }
@@ -589,6 +652,24 @@ __device__ __noinline__ void build_labels(uint32_t *tab, int k, int p) {
   constexpr int LS = P == 5 ? W * (R - 1) : (W * (R - 1) + 3) & ~3;
   const int np = (p - 1) / 2;
   uint32_t *lab = tab + k * (p - 1) * RWP;
+  if constexpr (log_labels(P, W)) {  // entry x: minus the logarithms (their complement), then the nonzero mask, per word
+    for (int x = threadIdx.x; x < k; x += kThreads) {
+      const uint32_t *e = tab + x * (p - 1) * RWP;
+      uint32_t *o = lab + x * RWP;
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        uint32_t cl[R - 1], l[R - 1];
+        fpbs::class_label<P, R>(e + w * R, cl, p);
+        fpbs::class_log<P, R>(cl, l);
+#pragma unroll
+        for (int i = 0; i + 1 < R; ++i) o[w * R + i] = ~l[i];
+        o[w * R + R - 1] = fpbs::nz<R>(e + w * R);
+      }
+#pragma unroll
+      for (int z = W * R; z < RWP; ++z) o[z] = 0u;
+    }
+    return;
+  }
   for (int i = threadIdx.x; i < k * np; i += kThreads) {
     const int t = i / np, q = i - t * np;
     const uint32_t *e = tab + (t * (p - 1) + q) * RWP;

@@ -94,12 +94,16 @@ FPK_HD int label_words(int p, int r, int W) { return p == 5 ? W * (r - 1) : (W *
 // Labels are kept while a lane's sum and its label leave room in 64
 // registers (beyond: spills), and while they fit behind the multiples.
 FPK_HD constexpr bool label_shape(int r, int W) { return W * (2 * r - 1) <= 36; }
+// p = 31 and 127 with at most 64 redundant positions (beyond: spills) keep
+// one entry a row instead: the logarithm of its class (fp_kernel.cuh).
+FPK_HD constexpr bool log_labels(int p, int W) { return (p == 31 || p == 127) && W <= 2; }
 // Words of an information set's labels; 0: none (p = 3 and 7 have row
 // signatures, and sets that would not fit take the two subtractions).
 FPK_HD int set_label_words(int p, int r, int W, int k) {
   if (p == 3 || p == 7 || !label_shape(r, W)) return 0;
-  const int words = k * ((p - 1) / 2) * label_words(p, r, W);
-  const int rows = k * (p - 1) * ((r * W + 3) & ~3);
+  const int rwp = (r * W + 3) & ~3;
+  const int words = log_labels(p, W) ? k * rwp : k * ((p - 1) / 2) * label_words(p, r, W);
+  const int rows = k * (p - 1) * rwp;
   return (rows + words) * 4 <= kSetBytesMax ? words : 0;
 }
 

@@ -22,11 +22,25 @@ def test_label_tells_classes_apart():
         assert cls[0] == {0}
 
 
-# n - k at one to four words and off their edges; (127, 30, 18), (251, 20, 9): labels do not fit behind the
+@pytest.mark.parametrize("p", [31, 127])
+def test_log_of_classes(p):
+    """3^(log s) is s or -s, and log s - log t is the class e with
+    s = +-3^e t (0 also as all ones): every pair of nonzero symbols."""
+    h = (p - 1) // 2
+    pairs = [(s, t) for s in range(1, p) for t in range(1, p)]
+    for i in range(0, len(pairs), 32):
+        ss, ts = zip(*pairs[i:i + 32])
+        logs, diffs = B.fpcode_test_class_log(p, ss, ts)
+        for s, t, a, d in zip(ss, ts, logs, diffs):
+            assert a < h and pow(3, a, p) in (s, p - s)
+            assert pow(3, d % h, p) * t % p in (s, p - s) and d <= h
+
+
+# n - k at one to four words and off their edges; (251, 20, 9): labels do not fit behind the
 # multiples; (61, 130, 4 and 6): a shape without labels
 CODES = [(5, 20, 5), (5, 45, 12), (5, 74, 10), (5, 104, 8), (5, 140, 12), (11, 30, 6), (13, 60, 6), (11, 100, 5),
-         (13, 133, 5), (17, 40, 5), (31, 24, 5), (31, 70, 6), (31, 100, 4), (31, 132, 4), (61, 40, 4), (61, 130, 4),
-         (127, 30, 3), (127, 70, 3), (127, 30, 18), (251, 20, 3), (251, 20, 9), (251, 60, 3), (61, 130, 6)]
+         (13, 133, 5), (17, 40, 5), (31, 24, 5), (31, 70, 6), (31, 42, 10), (31, 36, 4), (31, 100, 4), (31, 132, 4), (61, 40, 4), (61, 130, 4),
+         (127, 30, 3), (127, 70, 3), (127, 35, 3), (127, 66, 2), (127, 30, 18), (251, 20, 3), (251, 20, 9), (251, 60, 3), (61, 130, 6)]
 
 
 @pytest.mark.gpu
