@@ -210,7 +210,11 @@ int digit_bits(int p) { return digit_bits_of(p); }
 // taken as m = floor(n/k) full ones, and the passes of each round g summed
 // until the bound after the round, m (g + 1), reaches d.  Only a guide for
 // choosing the leaf form: the search itself certifies the true d.
-double expected_work_of(int p, int n, int k) {
+struct Expected {
+  double work;
+  int g;  // the last round
+};
+Expected expected_work_of(int p, int n, int k) {
   const double lq = std::log((double)p);
   double lsum = -1e300;
   int d = 1;
@@ -224,23 +228,25 @@ double expected_work_of(int p, int n, int k) {
   }
   const int m = std::max(1, n / k);
   double work = 0;
-  for (int g = 1; g <= k; ++g) {
+  int g = 1;
+  for (;; ++g) {
     work += m * std::exp(std::lgamma(k + 1.0) - std::lgamma(g + 1.0) - std::lgamma(k - g + 1.0) + (g - 1) * std::log(p - 1.0));
-    if (m * (g + 1) >= d) break;
+    if (m * (g + 1) >= d || g == k) break;
   }
-  return work;
+  return {work, g};
 }
 // The same, remembered per (p, n, k) by each thread (about fifty lgamma and
 // exp calls; a stream of codes of a few shapes asks for it once per shape).
-double expected_work(int p, int n, int k) {
-  thread_local std::unordered_map<uint32_t, double> memo;
+Expected expected_search(int p, int n, int k) {
+  thread_local std::unordered_map<uint32_t, Expected> memo;
   const uint32_t key = (uint32_t)p << 16 | (uint32_t)n << 8 | (uint32_t)k;
   auto it = memo.find(key);
   if (it != memo.end()) return it->second;
-  const double w = expected_work_of(p, n, k);
+  const Expected w = expected_work_of(p, n, k);
   if (memo.size() < 4096) memo.emplace(key, w);
   return w;
 }
+double expected_work(int p, int n, int k) { return expected_search(p, n, k).work; }
 // Tensor-core kernel (pair_leaves 2): from this much expected work on, and
 // with at least this many redundant symbols (its class comparison needs
 // some).  Measured, leaf kernels against it: F_7 [40,20] (4.2e7 codewords)
@@ -248,6 +254,20 @@ double expected_work(int p, int n, int k) {
 // 119 us, F_5 [51,24] (3.0e8) 431 against 126, F_7 [52,19] (2.9e10) 17 390
 // against 1 965.
 constexpr double kSplitWork = 1e8;
+// The same per pass: a pass on the tensor-core kernel costs some 5 us more in
+// hand-offs and tail tables, which a search of many small passes does not
+// get back.  Kernel times, leaf kernels against it, in order of the expected
+// codewords a pass: F_3 [80,22] (5e6) 105 and 131 us, [65,24] (1.1e7) 96 and
+// 127, F_5 [33,19] (1.5e7) 30 and 36; F_3 [85,25] (2.2e7) 309 and 273, [68,31]
+// (2.8e7) 77 and 57, [70,32] (3.6e7) 88 and 58.
+constexpr double kSplitPassWork = 1.8e7;
+bool split_pays(const Prepared &P, double total) {
+  const Expected x = expected_search(P.p, P.n, P.k);
+  size_t passes = 0;  // of the schedule, up to the expected last round
+  while (passes < P.passes.size() && P.passes[passes].g <= x.g) ++passes;
+  const double work = std::min(x.work, total);
+  return work >= kSplitWork && work >= kSplitPassWork * (double)passes;
+}
 constexpr int kSplitMinRed = 4;
 // Dynamic shared memory of one of its CTAs: 227 KiB less the kernel's own.
 constexpr int kSplitSmemMax = 218000;
@@ -497,7 +517,7 @@ int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prep
   P->split_k = P->split_nu = P->split_cap = 0;
   if (use != SplitUse::kNever && opts.pair_leaves == 2 && (p == 3 || p == 5 || p == 7) && k >= 3 &&
       n - k >= kSplitMinRed &&
-      (use == SplitUse::kAny || ((double)total >= kSplitWork && expected_work(p, n, k) >= kSplitWork))) {
+      (use == SplitUse::kAny || split_pays(*P, (double)total))) {
     const int K = fpk::split_k(p, n - k, &P->split_nu);
     if (K > 0) {
       const int room = kSplitSmemMax - fpk::split_off_tails(k, p, P->rwpad) - 256;

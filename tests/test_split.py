@@ -120,3 +120,13 @@ def test_split_search_equals_leaf_kernels(p, n, k, budget):
     assert np.array_equal(a.witness, b.witness)
     c = B.fpcode_min_distance_ex(pr, None, B.fpcode_opts_default(budget=budget))  # the same handle again, with early exits
     _same(c, b, ("status", "d", "L", "U", "m", "npasses", "counts", "kj"))
+
+
+@pytest.mark.parametrize("p,n,k,split", [(3, 80, 40, True), (3, 85, 25, True), (5, 51, 24, True), (7, 50, 25, True),
+                                         (3, 80, 22, False), (3, 65, 24, False), (5, 33, 19, False), (7, 40, 20, False)])
+def test_split_only_where_passes_are_large(p, n, k, split, lib):
+    """Many passes with little work each stay on the leaf kernels."""
+    code = inputs.single_code(60 + n, p, n, k)
+    pr = B.fpcode_prepare(p, n, k, code.G, B.fpcode_opts_default())
+    last = max(i for i, ps in enumerate(B.fpcode_prepared_schedule(pr)) if ps["g"] <= 3)
+    assert (B.fpcode_test_split_pass(pr, last, cap=1 << 16) is not None) is split
