@@ -309,7 +309,7 @@ int plan_one(fpcode_prepared *prep, const DevCtx &c) {
     fph::plan_split(&P, prep->ctas);
   else
     fph::plan_tasks(&P, prep->ctas, P.opts.prefixes_per_lane,
-                    P.opts.min_steps > 0 ? P.opts.min_steps : fph::kMinStepsSingle, true);
+                    std::max(0, P.opts.min_steps), true);
   if (prep->slice_hi > 0) {  // a slice of the one pass: its tasks under the same plan
     fpk::PassDesc &d = P.passes[0];
     const uint64_t hi = std::min<uint64_t>(prep->slice_hi, d.ntasks);

@@ -734,7 +734,13 @@ void plan_tasks(Prepared *P, int ctas, int fixed_pl, int min_steps, bool spread_
     // tasks of min_steps prefixes per lane on part of the grid, which takes
     // up the following passes meanwhile; a lane's setup (unranking its first
     // prefix, summing its rows) then serves several prefixes
-    const uint64_t umin = ((uint64_t)std::max(1, min_steps) + unit - 1) / unit;
+    uint64_t umin = ((uint64_t)(min_steps > 0 ? min_steps : kMinStepsSingle) + unit - 1) / unit;
+    // default of one code: where up to four units a lane fill the grid, all of
+    // it (kernel times, eight steps against the rule: F_3 [43,23] 38.7 and
+    // 28.5 us, F_31 [32,7] 43.0 and 35.7); F_7 [40,20] at six a lane instead
+    // of eight on two thirds of the grid took 46.7 us, not 45.0
+    const uint64_t fill = (N + lanes * C - 1) / (lanes * C);
+    if (min_steps <= 0 && fill <= 4) umin = std::min(umin, std::max<uint64_t>(1, fill));
     if (spread_tiny && N <= lanes * C) {  // under one unit per lane of the grid: spread it wide
       d.ntasks = (uint32_t)((N + lanes - 1) / lanes);
       continue;

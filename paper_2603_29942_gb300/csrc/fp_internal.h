@@ -94,7 +94,7 @@ int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prep
 // fixed_pl > 0: tasks of fixed_pl prefixes per lane everywhere.  Else a pass
 // too small to give every lane of the grid min_steps prefixes gets fixed
 // tasks of min_steps prefixes per lane (fewer tasks than CTAs), the others
-// guided tasks.  min_steps trades the latency of one small code (1: spread
+// guided tasks.  0: the default of one code, kMinStepsSingle or less.  min_steps trades the latency of one small code (1: spread
 // each pass over the whole grid) against throughput (a lane's setup cost
 // shared by more prefixes).  spread_tiny: a pass under one prefix unit per
 // lane of the grid still gets one unit per lane (the first passes of a
