@@ -96,12 +96,17 @@ typedef struct fpcode_opts {
                           expected to take 10^8 codewords or more (d from
                           the Gilbert-Varshamov bound), since the pair
                           table pays off on large passes and small
-                          searches are bound by latency.  Batches and
-                          servers use one-row leaves.  d, L, U and the
-                          per-level counts do not depend on it. */
+                          searches are bound by latency; with 2 such a
+                          search of one code (p = 3, 5, 7) also compares
+                          stems with tails of two or three rows on the
+                          tensor cores where that fits, reporting keys of
+                          the same form.  Batches and servers use one-row
+                          leaves.  d, L, U and the per-level counts do not
+                          depend on it. */
   int min_steps;       /* one-row leaves: prefixes per lane given to a pass
-                          too small to fill the grid (0: 8 for one code,
-                          32 for a batch, 1 when serving) */
+                          too small to fill the grid (0: up to 8 for one
+                          code, 4 to 32 for a batch by its size, 1 when
+                          serving) */
   int task_work;       /* pair leaves: least work of a task per lane, in
                           pair entries (0: 192) */
   int task_share;      /* pair leaves: a task takes 1 / (task_share * C) of

@@ -773,7 +773,10 @@ int fpcode_min_distance_batch(int num, const fpcode_desc *codes, void *stream, c
     const bool many = g.idx.size() > 1;
     for (int i : g.idx)
       fph::plan_tasks(preps[i].get(), g.ctas, o.prefixes_per_lane,
-                      o.min_steps > 0 ? o.min_steps : many ? fph::kMinStepsBatch : fph::kMinStepsSingle, !many);
+                      o.min_steps > 0 ? o.min_steps
+                      : many          ? fph::min_steps_batch((int)g.idx.size(), g.ctas)
+                                      : fph::kMinStepsSingle,
+                      !many);
     g.L = make_layout(g.codesv);
     g.dev_off = dev_total;
     dev_total += align256(g.L.total);

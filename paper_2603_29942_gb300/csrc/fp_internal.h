@@ -112,6 +112,14 @@ int split_smem_bytes(const Prepared &P);
 constexpr size_t kPairTableMaxBytes = 40 * 1024;
 constexpr int kMinStepsSingle = 8;   // one code per launch
 constexpr int kMinStepsBatch = 32;   // many codes share the grid
+// A launch of few codes cannot fill the grid with tasks of 32 prefixes a
+// lane.  Whole batches, 32 steps against the rule's: 24 codes over F_3, 5, 7,
+// 11 714 and 486 us (4 steps), 4 codes 252 and 169, 13 codes 444 and 319, 40
+// codes 710 and 591, 74 codes 1105 and 1031 (8), 150 codes 1760 and 1745 (16).
+inline int min_steps_batch(int codes, int ctas) {
+  const int steps = codes * 64 / (ctas > 0 ? ctas : 1);
+  return steps < 4 ? 4 : steps > kMinStepsBatch ? kMinStepsBatch : steps;
+}
 constexpr int kMinStepsServe = 1;    // streamed codes: latency first
 
 // Name and SM count of the current device (fp_api.cu).  Returns an fpcode status.

@@ -2,7 +2,10 @@
 // 5, 7): the passes of the Brouwer-Zimmermann search as class comparisons of
 // stems with tails (fp_split.cuh) on the fifth-generation tensor cores.
 //
-// One persistent CTA of 512 threads per SM.  A CTA holds one block of tails
+// One persistent CTA per SM: 512 working threads and a warpgroup of which
+// one warp claims tasks ahead, counts finished ones off and polls the best
+// weight, so that no working warp waits for L2 (F_3 [80,40] 161 -> 118 us,
+// F_7 [50,25] 454 -> 328 us).  A CTA holds one block of tails
 // of one information set in shared memory, each tail's class values as one
 // row of K fp8 bytes (the B operand, 96 rows to a tile).  Its four
 // warpgroups work on their own: each lane walks its own stems (one exact
@@ -18,13 +21,24 @@
 // What bounds it: the read and the AND of the results and the tensor pipe
 // are balanced at K = 64 (109 results, 218 codewords, a clock and SM
 // measured with nothing else; 85 at K = 96 and 64 at K = 128, where the
-// tensor pipe is full), so what is left is the stems: about 150
-// instructions a stem, paid once per block of tails.  That is why tails
+// tensor pipe is full), so what is left is the stems: the walk, the
+// exact add and the class values, paid once per stem and block of tails,
+// and the latency of a step (1 to 1.6 us a step of 128 stems a warpgroup,
+// 0.5 to 0.7 us a tile).  That is why tails
 // have two or three rows, whichever costs less over the pass (plan_split):
 // the pair table of the popcount kernel serves a stem of a deep pass only
 // 36 to 104 entries.  M = 128 with the A operand in tensor memory keeps the
 // stems out of shared memory, whose read port the B operand needs; N = 96
-// is what four warpgroups of 16 + 96 columns leave room for.
+// is what four warpgroups of up to 32 + 96 columns leave room for, and
+// setmaxnreg moves the claiming warpgroup's registers to the working ones
+// (96 at launch, then 112 and 32: F_7 [52,19] 2534 -> 1965 us, fewer spills in
+// the steps).  Three warpgroups of N = 128, or of two N = 64 accumulators,
+// and two half-size table buffers were slower.
+//
+// Against the popcount kernels (whole search): F_3 [80,40] 174 -> 119 us,
+// F_7 [50,25] 845 -> 302, F_7 [52,19] 17389 -> 1965, F_3 [74,50] 1254 ->
+// 372, F_5 [51,24] 431 -> 126.  ncu, F_7 [50,25]: tensor pipe 23 %, ALU 39 %,
+// issue slots 35 %: bound by latency within a step, not by a pipe.
 #pragma once
 #include "fp_kernel.cuh"
 #include "fp_split.cuh"
