@@ -71,12 +71,13 @@ PROBES = {"probe_f3_n80_k40_g8": ("f3_n80_k40", 8), "probe_f7_n40_k20_g7": ("f7_
 ADDITIONS = {"additions_f3": 3, "additions_f7": 7}
 FLUSH_BYTES = 256 << 20
 
-# DRAM bytes of one bz_kernel launch per workload, from one ncu capture of
+# DRAM bytes of one launch of the enumeration kernel per workload, from one ncu capture of
 # that workload (dram__bytes_read.sum + dram__bytes_write.sum, summarised
 # under profiles/).  Reported only while the kernel sources hash to the
 # version that was profiled; any later change of their code reports null
 # (the hash skips comments and blank lines).
-KERNEL_SOURCES = ["fp_kernel.cuh", "fp_enum.cuh", "fp_bitslice.cuh", "fp_types.h"]
+KERNEL_SOURCES = ["fp_kernel.cuh", "fp_enum.cuh", "fp_bitslice.cuh", "fp_types.h", "fp_split.cuh",
+                  "fp_split_kernel.cuh"]
 _SHA_PROFILED = "8780d0da516689b5a57dcd3df7282efb232c48e9f0263d9e0ea74675ba62254a"
 PROFILED_TRAFFIC: dict = {  # profiles/bz_kernel_*.md (the command of each capture is there)
     "f3_n80_k40": {"bytes": 5725952 + 0, "sources_sha256": _SHA_PROFILED},
@@ -104,6 +105,17 @@ def kernel_sources_sha256() -> str:
         with open(os.path.join(root, f), encoding="utf-8") as fh:
             h.update(code_of(fh.read()).encode())
     return h.hexdigest()
+
+
+def kernel_name(B, code) -> str:
+    """The kernel that searches the code under the default options."""
+    prep = B.fpcode_prepare(code.p, code.n, code.k, code.G, B.fpcode_opts_default())
+    second = next(i for i, ps in enumerate(B.fpcode_prepared_schedule(prep)) if ps["g"] >= 2)
+    try:
+        B.fpcode_test_split_runs(prep, second)
+    except B.FpcodeError:
+        return "bz_kernel"
+    return "split_kernel"
 
 
 def profiled_traffic(workload: str):
@@ -383,7 +395,7 @@ def probe_line(torch, B, code, name, g, d, stream, flush, peak_t, steps=5, warmu
     return {"bound": "alu", "achieved": ach, "peak": peak_t, "unit": "Tpopc/s", "frac": ach / peak_t,
             "traffic": profiled_traffic(name), "pass": [g, 0], "codewords": size, "kernel_ms": k_ms, "workload": name,
             "leaf_form": "pair" if B.fpcode_test_pair_mode(pr) else "one-row", "least_weight_in_pass": least,
-            "note": "the same kernel on one pass of fixed size alone, termination off, U seeded at d"}
+            "note": "bz_kernel on one pass of fixed size alone, termination off, U seeded at d"}
 
 
 def single_code(args, torch, B, name, stream, flush, world, clk_need=True):
@@ -545,7 +557,7 @@ def run_default(args, rank, world, local):
     W = head["W"]
     ach = head["codewords"] * W / (kern_ms * 1e-3) / 1e12
     roof = {"bound": "alu", "achieved": ach, "peak": peak["tpopc_s"], "unit": "Tpopc/s", "frac": ach / peak["tpopc_s"],
-            "traffic": profiled_traffic(args.workload), "kernel": "bz_kernel", "ops_per_codeword": W,
+            "traffic": profiled_traffic(args.workload), "kernel": kernel_name(B, head["code"]), "ops_per_codeword": W,
             "kernel_ms": kern_ms, "peak_basis": peak["basis"], "peak_of": "measured",
             "leaf_form": head["leaf_form"]}
     probe_of = {v[0]: (k, v[1]) for k, v in PROBES.items()}
