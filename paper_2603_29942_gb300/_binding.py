@@ -206,6 +206,7 @@ def _declare(lib):
         "fpcode_test_split_pass": (ctypes.c_int64, [_VP, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                     ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_uint64),
                                                     ctypes.c_int64]),
+        "fpcode_test_lose_products": (ctypes.c_int, [_VP, ctypes.c_int]),
         "fpcode_test_pair_table_device": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.POINTER(ctypes.c_uint32), ctypes.c_int]),
         "fpcode_prepared_pass_slice": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_uint64, ctypes.c_uint64, ctypes.c_int,
                                                       ctypes.POINTER(_VP)]),
@@ -877,6 +878,12 @@ def fpcode_test_split_pass(prep: Prepared, pass_index: int, ctas: int = 152, tai
     n = lib().fpcode_test_split_pass(prep.handle, int(pass_index), int(ctas), int(tail_rows), int(block), int(unit),
                                      int(esplit), keys.ctypes.data_as(ctypes.POINTER(ctypes.c_uint64)), cap)
     return None if n < 0 else keys[:min(n, cap)]
+
+
+def fpcode_test_lose_products(prep: Prepared, on: bool) -> None:
+    """One warpgroup's products of the tensor-core kernel never count as
+    complete in the searches that follow (on), until their wait gives up."""
+    _check(lib().fpcode_test_lose_products(prep.handle, int(on)), "fpcode_test_lose_products")
 
 
 def fpcode_test_split_runs(prep: Prepared, pass_index: int, ctas: int = 152) -> int:

@@ -393,7 +393,9 @@ int enqueue_one(fpcode_prepared *prep, cudaStream_t st, const fpcode_opts &o) {
   }
   if (!P.passes.empty()) {
     FP_CUDA(cudaEventRecord((cudaEvent_t)prep->ev0, st));
-    int s = launch(kernel_of(P), prep->ctas, prep->smem, st, prep->dev, L, kparams(o, 0), threads_of(P));
+    KParams kp = kparams(o, 0);
+    kp.lose = prep->lose;
+    int s = launch(kernel_of(P), prep->ctas, prep->smem, st, prep->dev, L, kp, threads_of(P));
     if (s) return s;
     FP_CUDA(cudaEventRecord((cudaEvent_t)prep->ev1, st));
   }
@@ -935,6 +937,12 @@ __global__ void intpeak_kernel(uint32_t *sink, long long *cycles, int iters, uin
 }  // namespace
 
 extern "C" {
+
+int fpcode_test_lose_products(fpcode_prepared *prep, int on) {
+  if (!prep || !prep->host.split) return FPCODE_EINVAL;
+  prep->lose = on ? 1 : 0;
+  return FPCODE_OK;
+}
 
 int fpcode_test_pass_times(fpcode_prepared *prep, void *stream, double *us, int max) {
   if (!prep || !prep->uploaded || !us) return -1;

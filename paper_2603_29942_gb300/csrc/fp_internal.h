@@ -145,6 +145,7 @@ struct fpcode_prepared {
   int device = -1;
   int ctas = 0;         // grid the tasks were planned for
   int smem = 0;         // dynamic shared memory of one launch
+  int lose = 0;         // test hook: KParams.lose of its launches
   int init_u = 0;       // > 0: the search starts with this upper bound (single-pass probes)
   int resume_from = 0;  // > 0: the next search starts at this pass (fpcode_search_resume)
   uint64_t slice_lo = 0, slice_hi = 0;  // slice_hi > 0: only tasks [slice_lo, slice_hi) of the one pass

@@ -65,6 +65,7 @@ struct KParams {
   unsigned long long idle_limit_ns;  // serving: exit after this long idle
   int32_t mid_pass;                  // -1: per code; 0 / 1: override
   int32_t lookahead;                 // 1: take tasks of later passes while earlier ones drain
+  int32_t lose;                      // test hook (split kernel): one warpgroup's products never count as come
 };
 
 // Launch-wide dynamic flags (zeroed before each launch).

@@ -75,17 +75,59 @@ __device__ __forceinline__ void mma_step(uint32_t d, uint32_t a, uint64_t b, uin
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-// Bounded: false if the barrier's phase never completed.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+               : "=r"(ok)
+               : "r"(bar), "r"(parity)
+               : "memory");
+  return ok != 0;
+}
+// Bounded: false if the barrier's phase has not completed after some thousand
+// tries (the caller goes on to wait_agreed).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < (1 << 20); ++i) {
-    uint32_t ok;
-    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(ok)
-                 : "r"(bar), "r"(parity)
-                 : "memory");
-    if (ok) return true;
-  }
+  for (int i = 0; i < (1 << 12); ++i)
+    if (mbar_test(bar, parity)) return true;
   return false;
+}
+// A wait that `warps` warps make for the same phase of a barrier, each of
+// them (in convergence): true once it has completed, false once the time of
+// all of them is up (`limit` ns, or at once when *over is set).  They leave
+// together or not at all: a warp that left alone would leave the others in
+// the named barriers that count on it.  Each of them comes here or sees the
+// phase complete, so the count of those whose time is up settles it: one that
+// sees the phase complete after all takes itself off the count, unless the
+// count is full.  `gave_up` starts at zero, and is of no use after a false.
+__device__ __noinline__ bool wait_agreed(uint32_t bar, uint32_t parity, unsigned long long limit, unsigned *gave_up,
+                                         unsigned warps, const int32_t *over) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const unsigned long long t0 = globaltimer();
+  for (;;) {
+    for (int i = 0; i < 256; ++i)
+      if (__all_sync(FULL, mbar_test(bar, parity))) return true;
+    int up = 0;
+    if (lane == 0) up = globaltimer() - t0 > limit || *(volatile const int32_t *)over;
+    if (__shfl_sync(FULL, up, 0)) break;
+  }
+  if (lane == 0) atomicAdd(gave_up, 1u);
+  const unsigned long long t1 = globaltimer();
+  for (;;) {
+    const bool came = __all_sync(FULL, mbar_test(bar, parity));
+    int leave = 0;  // 1: the phase is complete, 2: nobody waits for it any more
+    if (lane == 0) {
+      unsigned g = *(volatile unsigned *)gave_up;
+      while (came && !leave && g < warps) {
+        const unsigned was = atomicCAS(gave_up, g, g - 1u);
+        leave = was == g ? 1 : 0;
+        g = was;
+      }
+      // (the others' own limits end this; a limit all the same)
+      if (!leave && (g >= warps || globaltimer() - t1 > 2 * limit + 60000000000ull)) leave = 2;
+    }
+    leave = __shfl_sync(FULL, leave, 0);
+    if (leave) return leave == 1;
+  }
 }
 __device__ __forceinline__ void tmem_store8(uint32_t addr, const uint32_t (&v)[8]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr), "r"(v[0]),
@@ -271,7 +313,10 @@ struct SplitShared {
                                   // of its task (two, since the first warp may be a product ahead of the last)
   unsigned long long best_key;    // the code's best key (inverted) and finished flag, as the scheduler last read them
   int32_t finished;
-  int32_t failed;                 // a product never came: no more are issued
+  int32_t over;                   // the scheduler has given up a running task: nothing more is handed out
+  int32_t lost[kSplitGroups];     // a product of the warpgroup never came: it issues no more
+  unsigned gave_up[kSplitGroups + 1];  // warps whose wait for a product (last: for a task) has run out (wait_agreed)
+  unsigned long long wait_ns;     // longest wait for a product
   SlotState *states;              // of the launch
   SlotAux *aux;
   CtlDyn *cdyn;
@@ -445,7 +490,8 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
   // tails of the block above the run's first stem: as many tiles as any lane needs
   const int q0 = l > 0 && steps ? comb_floor(B, l - 1, k - t - 1, l, ncl, J0) : -1;
   const uint32_t tiles = (min(nb, tails_above(B, k, t, b, q0) - first) + kSplitN - 1) / kSplitN;
-  if (steps == 0 || slice >= tiles || *(volatile int32_t *)&sh.failed) {  // the same for the whole warpgroup
+  // the same for the whole warpgroup: its warps set `lost` themselves, and all of them before they left that task
+  if (steps == 0 || slice >= tiles || *(volatile int32_t *)&sh.lost[grp]) {
     nearly();
     return 0;
   }
@@ -543,9 +589,15 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
       } else {
         group_arrive(1 + grp);
       }
-      if (!__all_sync(FULL, mbar_wait(mbar, parity))) {  // never seen: reported as a timeout; nothing more is issued
-        *(volatile int32_t *)&sh.failed = 1;
-        atomicExch(&sh.cdyn->err, 1);
+      if (!__all_sync(FULL, mbar_wait(mbar, parity)) &&
+          !wait_agreed(mbar, parity, sh.wait_ns, &sh.gave_up[grp], kSplitGroup / 32, &sh.over)) {
+        // never seen, by any warp of the group: reported as a timeout
+        if (lane == 0) {
+          *(volatile int32_t *)&sh.lost[grp] = 1;
+          atomicExch(&sh.cdyn->err, 1);
+        }
+        __syncwarp();
+        if (i + 1 < steps) nearly();
         return 0;
       }
       stop = *(volatile int32_t *)&sh.stop[grp][parity];
@@ -595,24 +647,6 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
   return (unsigned long long)seen << (l > 0 ? 1 : 0);
 }
 
-// Waits bounded by time (globaltimer looked at now and then).
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-               : "=r"(ok)
-               : "r"(bar), "r"(parity)
-               : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait_ns(uint32_t bar, uint32_t parity, unsigned long long limit) {
-  if (mbar_test(bar, parity)) return true;
-  const unsigned long long t0 = globaltimer();
-  for (;;) {
-    for (int i = 0; i < 256; ++i)
-      if (mbar_test(bar, parity)) return true;
-    if (globaltimer() - t0 > limit) return false;
-  }
-}
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -653,14 +687,18 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int i = 0; i < kSplitGroups; ++i) mbar_init(smem_u32(&s_sh.product[i]), 1);
+    // (a test has the first warpgroup of CTA 0 wait for an arrival that nobody makes)
+    for (int i = 0; i < kSplitGroups; ++i) mbar_init(smem_u32(&s_sh.product[i]), kp.lose && blockIdx.x == 0 && i == 0 ? 2 : 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&s_sh.full[i]), 1);
       mbar_init(smem_u32(&s_sh.near[i]), kSplitGroups);
       mbar_init(smem_u32(&s_sh.done[i]), kSplitWarps);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    s_sh.failed = 0;
+    s_sh.over = 0;
+    for (int i = 0; i < kSplitGroups; ++i) s_sh.lost[i] = 0;
+    for (int i = 0; i <= kSplitGroups; ++i) s_sh.gave_up[i] = 0;
+    s_sh.wait_ns = kp.wait_limit_ns;
     s_sh.best_key = 0;
     s_sh.finished = 0;
     s_sh.states = states;
@@ -717,7 +755,7 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
       }
       uint32_t head = 0, tail = 0;  // tasks handed out, tasks counted off
       unsigned long long since = 0;  // when the scheduler began to wait for a running task
-      bool over = false;
+      bool over = false, stuck = false;
       for (;;) {
         if (!over && head - tail < 2) {
           // one task runs: the next is claimed once its warpgroups are in their last steps
@@ -778,13 +816,18 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
           since = globaltimer();
         } else if (globaltimer() - since > wait_ns) {
           atomicExch(&cdyn->err, 1);  // a warp never finished: report a timeout
+          stuck = true;
           break;
         } else {
           __nanosleep(200);  // the issue slots belong to the warps that work
         }
       }
-      s_sh.task[head & 1u].cmd = kCmdExit;
-      mbar_arrive(smem_u32(&s_sh.full[head & 1u]));
+      if (stuck && head - tail == 2) {  // both buffers hold tasks that are not counted off
+        *(volatile int32_t *)&s_sh.over = 1;
+      } else {
+        s_sh.task[head & 1u].cmd = kCmdExit;
+        mbar_arrive(smem_u32(&s_sh.full[head & 1u]));
+      }
     }
     __syncwarp();
   } else {
@@ -797,11 +840,11 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
     for (uint32_t n = 0;; ++n) {
       const int b = (int)(n & 1u);
       SplitTask &tk = s_sh.task[b];
-      if (!mbar_wait_ns(smem_u32(&s_sh.full[n & 1u]), (n >> 1) & 1u, wait_ns)) {
+      if (!wait_agreed(smem_u32(&s_sh.full[n & 1u]), (n >> 1) & 1u, wait_ns, &s_sh.gave_up[kSplitGroups], kSplitWarps,
+                       &s_sh.over)) {  // no warp has anything more to wait for
         atomicExch(&cdyn->err, 1);
         break;
       }
-      __syncwarp();
       if (tk.cmd == kCmdExit) break;
       if (tk.stage || tk.build) {
         if (tid == 0) tk.drop = *(volatile int32_t *)&s_sh.finished;

@@ -1,0 +1,32 @@
+"""What the tensor-core kernel does when a product never counts as complete:
+its waits end, and the launch leaves a usable handle behind."""
+import time
+
+import pytest
+
+from paper_2603_29942_gb300 import _binding as B
+from paper_2603_29942_gb300 import inputs
+
+
+def _same(a, b):
+    for f in ("status", "d", "L", "U", "m", "npasses", "counts", "kj", "best_key", "enumerated"):
+        assert getattr(a, f) == getattr(b, f), f
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("p,n,k,budget", [(3, 80, 40, 0), (7, 52, 19, 3 * 10 ** 8), (5, 40, 20, 0)])
+def test_lost_product_ends_the_launch(p, n, k, budget):
+    """One warpgroup waits for an arrival that nobody makes: it gives up as a
+    whole after the wait limit, the other warps of its CTA are not left in a
+    barrier, and the same handle then gives the same result as before."""
+    code = inputs.single_code(400 + n, p, n, k)
+    o = B.fpcode_opts_default(budget=budget, mid_pass_exit=0, wait_limit_s=0.05)
+    pr = B.fpcode_test_prepare_split(p, n, k, code.G, o)
+    before = B.fpcode_min_distance_ex(pr, None, o)
+    B.fpcode_test_lose_products(pr, True)
+    t0 = time.time()
+    for _ in range(2):
+        B.fpcode_min_distance_ex(pr, None, o)
+    assert time.time() - t0 < 20
+    B.fpcode_test_lose_products(pr, False)
+    _same(B.fpcode_min_distance_ex(pr, None, o), before)
