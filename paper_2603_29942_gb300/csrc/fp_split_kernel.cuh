@@ -314,6 +314,7 @@ struct SplitShared {
   unsigned long long best_key;    // the code's best key (inverted) and finished flag, as the scheduler last read them
   int32_t finished;
   int32_t over;                   // the scheduler has given up a running task: nothing more is handed out
+  int32_t lost_any;               // ... or a warpgroup has lost a product
   int32_t lost[kSplitGroups];     // a product of the warpgroup never came: it issues no more
   unsigned gave_up[kSplitGroups + 1];  // warps whose wait for a product (last: for a task) has run out (wait_agreed)
   unsigned long long wait_ns;     // longest wait for a product
@@ -594,6 +595,7 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
         // never seen, by any warp of the group: reported as a timeout
         if (lane == 0) {
           *(volatile int32_t *)&sh.lost[grp] = 1;
+          *(volatile int32_t *)&sh.lost_any = 1;
           atomicExch(&sh.cdyn->err, 1);
         }
         __syncwarp();
@@ -687,15 +689,15 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    // (a test has the first warpgroup of CTA 0 wait for an arrival that nobody makes)
-    for (int i = 0; i < kSplitGroups; ++i) mbar_init(smem_u32(&s_sh.product[i]), kp.lose && blockIdx.x == 0 && i == 0 ? 2 : 1);
+    // (a test has the first warpgroup wait for an arrival that nobody makes)
+    for (int i = 0; i < kSplitGroups; ++i) mbar_init(smem_u32(&s_sh.product[i]), kp.lose && i == 0 ? 2 : 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&s_sh.full[i]), 1);
       mbar_init(smem_u32(&s_sh.near[i]), kSplitGroups);
       mbar_init(smem_u32(&s_sh.done[i]), kSplitWarps);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    s_sh.over = 0;
+    s_sh.over = s_sh.lost_any = 0;
     for (int i = 0; i < kSplitGroups; ++i) s_sh.lost[i] = 0;
     for (int i = 0; i <= kSplitGroups; ++i) s_sh.gave_up[i] = 0;
     s_sh.wait_ns = kp.wait_limit_ns;
@@ -804,6 +806,10 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
         }
         if (mbar_test(smem_u32(&s_sh.done[o]), op)) {
           const SplitTask &tk = s_sh.task[o];
+          // A lost product: some of the task's codewords were never compared.
+          // It is not counted off, so its pass never counts as complete and
+          // the search ends as a timeout, unless an earlier pass certifies.
+          if (*(volatile int32_t *)&s_sh.lost_any) break;
           if (tk.count) {
             atomicAdd(&states[0].enumerated, tk.count);
             atomicAdd(&cs.aux->pass_count[tk.cl.pass], tk.count);

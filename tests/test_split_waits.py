@@ -30,3 +30,18 @@ def test_lost_product_ends_the_launch(p, n, k, budget):
     assert time.time() - t0 < 20
     B.fpcode_test_lose_products(pr, False)
     _same(B.fpcode_min_distance_ex(pr, None, o), before)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("p,n,k,budget", [(3, 80, 40, 0), (7, 52, 19, 3 * 10 ** 8), (5, 40, 20, 0)])
+def test_lost_product_is_a_timeout(p, n, k, budget):
+    """A task that was not compared in full is not counted off: the search
+    reports a timeout, certifies nothing and claims no distance."""
+    code = inputs.single_code(400 + n, p, n, k)
+    o = B.fpcode_opts_default(budget=budget, mid_pass_exit=0, wait_limit_s=0.05)
+    pr = B.fpcode_test_prepare_split(p, n, k, code.G, o)
+    whole = B.fpcode_min_distance_ex(pr, None, o)
+    B.fpcode_test_lose_products(pr, True)
+    r = B.fpcode_min_distance_ex(pr, None, o)
+    assert r.status == B.ETIMEOUT and r.d == -1
+    assert r.L <= whole.L and r.U >= whole.U
