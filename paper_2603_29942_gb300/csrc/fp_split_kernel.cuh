@@ -462,7 +462,8 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
     // pass the threshold anyway)
     nearly();
     if (l > 0 && steps) stem_start<P, R, W, DB>(x, mult, B, u0, k, t, l, ncl);
-    for (uint32_t i = 0; i < steps && !finished(); ++i) {
+    // (one lane's read of the flag for the warp: it changes meanwhile, and the body's collectives take all lanes)
+    for (uint32_t i = 0; i < steps && !__shfl_sync(FULL, finished(), 0); ++i) {
       if (l > 0 && i) stem_next<P, R, W, DB>(x, mult, l);
       const uint32_t E = min(nb, tails_above(B, k, t, b, x.pos.m) - first);
       take_up();

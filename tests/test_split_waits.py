@@ -45,3 +45,19 @@ def test_lost_product_is_a_timeout(p, n, k, budget):
     r = B.fpcode_min_distance_ex(pr, None, o)
     assert r.status == B.ETIMEOUT and r.d == -1
     assert r.L <= whole.L and r.U >= whole.U
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("p,n,k", [(3, 80, 40), (7, 40, 20), (5, 51, 24)])
+def test_search_that_ends_inside_direct_passes(p, n, k):
+    """A code with a codeword of weight 1 certifies with its first pass, while
+    other CTAs walk stems of the passes after it with every weight exact: the
+    finished flag reaches them in the middle, 200 times over."""
+    code = inputs.single_code(500 + n, p, n, k)
+    G = code.G.copy()
+    G[0, k:] = 0
+    o = B.fpcode_opts_default()
+    pr = B.fpcode_test_prepare_split(p, n, k, G, o)
+    for _ in range(200):
+        r = B.fpcode_min_distance_ex(pr, None, o)
+        assert r.status == B.OK and r.d == 1 and r.enumerated == sum(r.counts)
