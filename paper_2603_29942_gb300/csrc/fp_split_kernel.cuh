@@ -75,6 +75,12 @@ __device__ __forceinline__ void mma_step(uint32_t d, uint32_t a, uint64_t b, uin
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
@@ -325,6 +331,7 @@ struct SplitShared {
   SplitTask task[2];              // the one that runs and the next one
   // mbarriers: of each task buffer, full (1 arrival), near its end (one per
   // warpgroup) and done (one per warp); of each warpgroup, its products
+  // (the commit's arrival and the issuing warp's)
   unsigned long long full[2], near[2], done[2], product[kSplitGroups];
 };
 
@@ -576,7 +583,10 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
     for (uint32_t c = slice; c < tiles && !stop; c += slices) {
       tc_before_sync();
       if ((warp & 3) == 0) {
-        if (lane == 0) *(volatile int32_t *)&sh.stop[grp][parity] = finished();
+        if (lane == 0) {
+          *(volatile int32_t *)&sh.stop[grp][parity] = finished();
+          mbar_arrive(mbar);  // the product's barrier takes this release and the commit: who sees it sees `stop`
+        }
         group_sync(1 + grp);
         tc_after_sync();
         if (elect_one()) {
@@ -650,12 +660,6 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
   return (unsigned long long)seen << (l > 0 ? 1 : 0);
 }
 
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 __device__ __forceinline__ void workers_sync() { asm volatile("bar.sync 5, %0;" ::"n"(kSplitThreads) : "memory"); }
 
 // The kernel: claims, counts and termination tests follow bz_kernel's
@@ -691,7 +695,7 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
   }
   if (tid == 0) {
     // (a test has the first warpgroup wait for an arrival that nobody makes)
-    for (int i = 0; i < kSplitGroups; ++i) mbar_init(smem_u32(&s_sh.product[i]), kp.lose && i == 0 ? 2 : 1);
+    for (int i = 0; i < kSplitGroups; ++i) mbar_init(smem_u32(&s_sh.product[i]), kp.lose && i == 0 ? 3 : 2);
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&s_sh.full[i]), 1);
       mbar_init(smem_u32(&s_sh.near[i]), kSplitGroups);
