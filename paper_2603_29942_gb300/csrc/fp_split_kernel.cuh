@@ -883,6 +883,7 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
+      __syncwarp();  // lane 0 arrives for the records of all lanes
       if ((tid & 31) == 0) {
         if (count) atomicAdd(&tk.count, count);
         mbar_arrive(smem_u32(&s_sh.done[b]));
