@@ -111,13 +111,28 @@ const void *kernel_for(int variant) {
   }
 }
 
+// Let `fn` be launched with `smem` bytes of dynamic shared memory.  The limit
+// belongs to the function, which every handle and thread shares: once a code
+// needs the opt-in (dynamic and static together past 48 KiB), it is raised to
+// all that the device allows, and never set to one code's size (a smaller code
+// prepared later would have the larger one's launches refused).
+int allow_smem(const void *fn, size_t smem, cudaFuncAttributes *fa) {
+  FP_CUDA(cudaFuncGetAttributes(fa, fn));
+  if (smem + fa->sharedSizeBytes <= 48 * 1024) return FPCODE_OK;
+  int dev = 0, most = 0;
+  FP_CUDA(cudaGetDevice(&dev));
+  FP_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  most -= (int)fa->sharedSizeBytes;
+  if (fa->maxDynamicSharedSizeBytes < most)
+    FP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+  return FPCODE_OK;
+}
+
 // CTAs per SM for a kernel with `smem` bytes of dynamic shared memory.
 int occupancy(const void *fn, int smem, int override_per_sm, int *per_sm, int threads) {
   cudaFuncAttributes fa{};
-  FP_CUDA(cudaFuncGetAttributes(&fa, fn));
-  // dynamic and static shared memory together past 48 KiB need the opt-in
-  if ((size_t)smem + fa.sharedSizeBytes > 48 * 1024)
-    FP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  const int s = allow_smem(fn, (size_t)smem, &fa);
+  if (s) return s;
   int n = 0;
   FP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, threads, (size_t)smem));
   if (n < 1) {
@@ -969,7 +984,8 @@ int fpcode_test_pair_table_device(const fpcode_prepared *prep, int j, uint32_t *
   cudaError_t e = cudaMalloc(&d_rows, mw * 4);
   if (e == cudaSuccess) e = cudaMalloc(&d_out, (size_t)words * 4 + 4);
   if (e == cudaSuccess) e = cudaMemcpy(d_rows, &P->table[(size_t)j * mw], mw * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && smem > 48 * 1024) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaFuncAttributes fa{};
+  if (e == cudaSuccess && fpd::allow_smem(fn, (size_t)smem, &fa)) e = cudaErrorInvalidValue;
   if (e == cudaSuccess) {
     const uint32_t *rows = d_rows;
     int k = P->k, rwpad = P->rwpad, sigp = P->pair_sigp, ow = words;
