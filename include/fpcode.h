@@ -67,8 +67,11 @@ typedef struct fpcode_opts {
                           earlier), catching up its levels 1..g */
   int mid_pass_exit;   /* 1 (default): stop a pass as soon as U <= L held
                           before it (early termination, Sec. 4.4); d and the
-                          per-level counts are unchanged, `enumerated` and
-                          the choice among equal-weight witnesses may vary */
+                          per-level counts are unchanged, `enumerated` (the
+                          tasks of the last pass that had begun when the
+                          record that ends it was found) and the choice
+                          among equal-weight witnesses may vary from run
+                          to run */
   int ctas_per_sm;     /* 0: from the occupancy calculator */
   int prefixes_per_lane; /* one-row leaves: 0: the task plan (guided
                           tasks, min_steps for small passes); else fixed
