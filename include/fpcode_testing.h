@@ -130,6 +130,9 @@ int fpcode_test_prepare_split(int p, int n, int k, const uint8_t *G, const fpcod
  * written), or -1 (no such pass, or the code is not searched this way). */
 int64_t fpcode_test_split_pass(fpcode_prepared *prep, int pass, int ctas, int tail_rows, int block, int unit, int esplit,
                                uint64_t *keys, int64_t max);
+/* 1 if a claim that finds a slot's task counter at `word`, past every task
+ * of its code, marks the code used up (serving: slot scans skip it). */
+int fpcode_test_marks_used_up(uint64_t word);
 /* Searches of `prep` from now on (on != 0) run with one warpgroup of
  * each CTA of the tensor-core kernel waiting for a product that never counts as complete,
  * until its wait limit (fpcode_opts.wait_limit_s) has passed: nothing is left

@@ -206,6 +206,7 @@ def _declare(lib):
         "fpcode_test_split_pass": (ctypes.c_int64, [_VP, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                     ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_uint64),
                                                     ctypes.c_int64]),
+        "fpcode_test_marks_used_up": (ctypes.c_int, [ctypes.c_uint64]),
         "fpcode_test_lose_products": (ctypes.c_int, [_VP, ctypes.c_int]),
         "fpcode_test_pair_table_device": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.POINTER(ctypes.c_uint32), ctypes.c_int]),
         "fpcode_prepared_pass_slice": (ctypes.c_int, [_VP, ctypes.c_int, ctypes.c_uint64, ctypes.c_uint64, ctypes.c_int,

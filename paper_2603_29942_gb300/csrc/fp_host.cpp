@@ -1393,6 +1393,8 @@ int64_t fpcode_test_split_pass(fpcode_prepared *prep, int pass, int ctas, int ta
   return n;
 }
 
+int fpcode_test_marks_used_up(uint64_t word) { return fpk::marks_used_up(word) ? 1 : 0; }
+
 int fpcode_prepared_shape(const fpcode_prepared *prep, int *m, int *kj, int *npasses, int *complete) {
   const fph::Prepared *P = prep ? &prep->host : nullptr;
   if (!P) return FPCODE_EINVAL;

@@ -1155,8 +1155,10 @@ __device__ __forceinline__ bool locate(ClaimCache &cc, const PassDesc *pc, int n
   return true;
 }
 
-// Mark the slot's task sequence used up, for the code of generation gen only.
-__device__ __forceinline__ void mark_exhausted(const CtlStatic &cs, int s, unsigned long long gen) {
+// Mark the slot's task sequence used up, for the code of generation gen only;
+// w: its task counter, which `locate` found past the last task.
+__device__ __forceinline__ void mark_exhausted(const CtlStatic &cs, int s, unsigned long long gen, unsigned long long w) {
+  if (!marks_used_up(w)) return;
   const uint32_t g = slot_flag_gen(gen);
   atomicCAS(&cs.slot_flags[s], g, g | kSlotExhausted);
 }
@@ -1313,7 +1315,7 @@ __device__ __forceinline__ int claim(const SlotDesc *slots, SlotState *states, c
     }
     if ((w >> kGenShift) == cc.gen && cc.sd.npasses > 0 && fin != fin_tag(cc.gen)) {
       if (locate(cc, pc, npc, w & kTaskMask)) got = s;
-      else mark_exhausted(cs, s, cc.gen);
+      else mark_exhausted(cs, s, cc.gen, w);
     }
     if (got < 0) slot_leave(cs, s);
   }
@@ -1343,7 +1345,7 @@ __device__ __forceinline__ int claim(const SlotDesc *slots, SlotState *states, c
       live = true;
       if (wgen != cc.gen) continue;  // slot in transition between two codes
       if (!locate(cc, pc, cc.slot == 0 ? npc : 0, w & kTaskMask)) {  // every task handed out
-        mark_exhausted(cs, s, wgen);
+        mark_exhausted(cs, s, wgen, w);
         continue;
       }
       if (!kp.lookahead && cc.P > ld_vol(&st->frontier)) continue;  // one pass at a time
@@ -1360,7 +1362,7 @@ __device__ __forceinline__ int claim(const SlotDesc *slots, SlotState *states, c
         }
       }
       if (!locate(cc, pc, cc.slot == 0 ? npc : 0, w & kTaskMask)) {
-        mark_exhausted(cs, s, cc.gen);
+        mark_exhausted(cs, s, cc.gen, w);
         slot_leave(cs, s);
         continue;
       }

@@ -61,8 +61,9 @@ constexpr size_t kServeTableCode = 256 * 1024;    // largest table of one code
 // reaches, so claims that read it find nothing to do and never wrap into a
 // real index), then the rest of the fresh state, then the counter at task
 // 0, then the slot's flag word.  A claim therefore never sees a claimable
-// counter next to a state that is still being written.
-constexpr uint64_t kTaskTransit = 1ull << 39;
+// counter next to a state that is still being written, and one that meets the
+// transition value leaves the slot's flag word alone (fpk::marks_used_up).
+using fpk::kTaskTransit;
 
 struct Slot {
   bool busy = false;

@@ -329,6 +329,16 @@ constexpr int32_t kRunning = -1;
 constexpr uint64_t kTaskMask = (1ull << 40) - 1;
 constexpr int kGenShift = 48;
 constexpr uint64_t kGenMask = 0xFFFFull;
+// Serving: task index of the counter while the host writes the next code
+// into the slot (past every schedule's tasks, claims on top of it included).
+constexpr uint64_t kTaskTransit = 1ull << 39;
+// Whether a claim that found the counter past the code's tasks may mark the
+// slot used up: not at the transition value or claims on top of it, when no
+// task has been handed out yet.  (The flag word is the last thing the host
+// writes, but a fence and several loads lie between a claim's read of the
+// counter and its mark: the mark could still fall on the new flag word, and a
+// code that has not begun would be skipped by every slot scan.)
+FPK_HD bool marks_used_up(uint64_t word) { return (word & kTaskMask) < kTaskTransit; }
 
 // SlotState.finished of a concluded code: its generation in the high half,
 // so that a claim of the next code in the slot never reads a predecessor's
