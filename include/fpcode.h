@@ -103,7 +103,10 @@ typedef struct fpcode_opts {
                           search of one code (p = 3, 5, 7) also compares
                           stems with tails of two or three rows on the
                           tensor cores where that fits, reporting keys of
-                          the same form.  Batches and servers use one-row
+                          the same form, unless a size of the leaf kernels'
+                          tasks is asked for (prefixes_per_lane, min_steps,
+                          task_work or task_share above 0); it has one CTA
+                          per SM whatever ctas_per_sm.  Batches and servers use one-row
                           leaves.  d, L, U and the per-level counts do not
                           depend on it. */
   int min_steps;       /* one-row leaves: prefixes per lane given to a pass

@@ -509,13 +509,15 @@ int prepare(int p, int n, int k, const uint8_t *G, const fpcode_opts &opts, Prep
     if (P->passes.size() > round_start && !truncated) P->passes.back().round_end = 1;
   }
   P->complete = truncated ? 0 : 1;
-  // The tensor-core kernel takes the code when the leaf form is left to the
-  // library, its class values fit a row, a useful number of tails fits
-  // beside them, and the search is large: expected to be, and not cut short
-  // by its budget.
+  // The tensor-core kernel takes the code when the leaf form and the task
+  // plan are left to the library (its plan has no use for the leaf kernels'
+  // task sizes: a caller who sets one gets the kernel that it is for), its
+  // class values fit a row, a useful number of tails fits beside them, and the
+  // search is large: expected to be, and not cut short by its budget.
+  const bool leaf_plan = opts.prefixes_per_lane > 0 || opts.min_steps > 0 || opts.task_work > 0 || opts.task_share > 0;
   P->split = false;
   P->split_k = P->split_nu = P->split_cap = 0;
-  if (use != SplitUse::kNever && opts.pair_leaves == 2 && (p == 3 || p == 5 || p == 7) && k >= 3 &&
+  if (use != SplitUse::kNever && opts.pair_leaves == 2 && !leaf_plan && (p == 3 || p == 5 || p == 7) && k >= 3 &&
       n - k >= kSplitMinRed &&
       (use == SplitUse::kAny || split_pays(*P, (double)total))) {
     const int K = fpk::split_k(p, n - k, &P->split_nu);
