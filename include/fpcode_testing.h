@@ -135,8 +135,8 @@ int64_t fpcode_test_split_pass(fpcode_prepared *prep, int pass, int ctas, int ta
 int fpcode_test_marks_used_up(uint64_t word);
 /* Searches of `prep` from now on (on != 0) run with one warpgroup of
  * each CTA of the tensor-core kernel waiting for a product that never counts as complete,
- * until its wait limit (fpcode_opts.wait_limit_s) has passed: nothing is left
- * out or in flight, one barrier only expects an arrival that nobody makes.
+ * until its wait runs out (about a second): nothing is left out or in flight,
+ * one barrier only expects an arrival that nobody makes.
  * FPCODE_EINVAL if that kernel does not search the code. */
 int fpcode_test_lose_products(fpcode_prepared *prep, int on);
 /* Microseconds from the start of the last search on `prep` to the end of

@@ -60,6 +60,8 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void tc_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
+constexpr int kCloseBar = 6;  // named barriers: 1 .. 4 the warpgroups' products, 5 the working warps, 6 .. 9 the warpgroups' closes
+constexpr int kLost = 2;
 __device__ __forceinline__ void group_arrive(int id) { asm volatile("bar.arrive %0, 128;" ::"r"(id) : "memory"); }
 
 // D (f16, 128 x N, tensor memory) = (accumulate ? D : 0) + A (e4m3, tensor memory) B^T (e4m3, shared memory)
@@ -89,51 +91,11 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
                : "memory");
   return ok != 0;
 }
-// Bounded: false if the barrier's phase has not completed after some thousand
-// tries (the caller goes on to wait_agreed).
+// Bounded: false if the barrier's phase has not completed after 2^18 tries (about a second).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < (1 << 12); ++i)
+  for (int i = 0; i < (1 << 18); ++i)
     if (mbar_test(bar, parity)) return true;
   return false;
-}
-// A wait that `warps` warps make for the same phase of a barrier, each of
-// them (in convergence): true once it has completed, false once the time of
-// all of them is up (`limit` ns, or at once when *over is set).  They leave
-// together or not at all: a warp that left alone would leave the others in
-// the named barriers that count on it.  Each of them comes here or sees the
-// phase complete, so the count of those whose time is up settles it: one that
-// sees the phase complete after all takes itself off the count, unless the
-// count is full.  `gave_up` starts at zero, and is of no use after a false.
-__device__ __noinline__ bool wait_agreed(uint32_t bar, uint32_t parity, unsigned long long limit, unsigned *gave_up,
-                                         unsigned warps, const int32_t *over) {
-  constexpr unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const unsigned long long t0 = globaltimer();
-  for (;;) {
-    for (int i = 0; i < 256; ++i)
-      if (__all_sync(FULL, mbar_test(bar, parity))) return true;
-    int up = 0;
-    if (lane == 0) up = globaltimer() - t0 > limit || *(volatile const int32_t *)over;
-    if (__shfl_sync(FULL, up, 0)) break;
-  }
-  if (lane == 0) atomicAdd(gave_up, 1u);
-  const unsigned long long t1 = globaltimer();
-  for (;;) {
-    const bool came = __all_sync(FULL, mbar_test(bar, parity));
-    int leave = 0;  // 1: the phase is complete, 2: nobody waits for it any more
-    if (lane == 0) {
-      unsigned g = *(volatile unsigned *)gave_up;
-      while (came && !leave && g < warps) {
-        const unsigned was = atomicCAS(gave_up, g, g - 1u);
-        leave = was == g ? 1 : 0;
-        g = was;
-      }
-      // (the others' own limits end this; a limit all the same)
-      if (!leave && (g >= warps || globaltimer() - t1 > 2 * limit + 60000000000ull)) leave = 2;
-    }
-    leave = __shfl_sync(FULL, leave, 0);
-    if (leave) return leave == 1;
-  }
 }
 __device__ __forceinline__ void tmem_store8(uint32_t addr, const uint32_t (&v)[8]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr), "r"(v[0]),
@@ -322,8 +284,6 @@ struct SplitShared {
   int32_t over;                   // the scheduler has given up a running task: nothing more is handed out
   int32_t lost_any;               // ... or a warpgroup has lost a product
   int32_t lost[kSplitGroups];     // a product of the warpgroup never came: it issues no more
-  unsigned gave_up[kSplitGroups + 1];  // warps whose wait for a product (last: for a task) has run out (wait_agreed)
-  unsigned long long wait_ns;     // longest wait for a product
   SlotState *states;              // of the launch
   SlotAux *aux;
   CtlDyn *cdyn;
@@ -499,11 +459,12 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
   // tails of the block above the run's first stem: as many tiles as any lane needs
   const int q0 = l > 0 && steps ? comb_floor(B, l - 1, k - t - 1, l, ncl, J0) : -1;
   const uint32_t tiles = (min(nb, tails_above(B, k, t, b, q0) - first) + kSplitN - 1) / kSplitN;
-  // the same for the whole warpgroup: its warps set `lost` themselves, and all of them before they left that task
+  // the same for the whole warpgroup: `lost` as of the close of an earlier task
   if (steps == 0 || slice >= tiles || *(volatile int32_t *)&sh.lost[grp]) {
     nearly();
     return 0;
   }
+  int stop = 0;  // the code has finished, or (kLost) a product never came
   for (uint32_t i = 0; i < steps; ++i) {
     if (i + 1 == steps) nearly();
     const bool act = i < nst;
@@ -579,14 +540,9 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
         }
       } while (any);
     };
-    int stop = 0;
     for (uint32_t c = slice; c < tiles && !stop; c += slices) {
       tc_before_sync();
       if ((warp & 3) == 0) {
-        if (lane == 0) {
-          *(volatile int32_t *)&sh.stop[grp][parity] = finished();
-          mbar_arrive(mbar);  // the product's barrier takes this release and the commit: who sees it sees `stop`
-        }
         group_sync(1 + grp);
         tc_after_sync();
         if (elect_one()) {
@@ -596,22 +552,20 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
           if (K > 64) mma_step<true>(tD, tA + 16, d0 + 32, kSplitIdesc);
           if (K > 96) mma_step<true>(tD, tA + 24, d0 + 48, kSplitIdesc);
           mma_commit(mbar);
+          // the product's barrier takes the commit and this release: who sees its
+          // phase sees `stop` (written after the group's barrier, so of a warp
+          // that has given up an earlier product too; ahead of that barrier the
+          // release cost F_3 [74,50] 12 %)
+          *(volatile int32_t *)&sh.stop[grp][parity] = finished() | *(volatile int32_t *)&sh.lost[grp];
+          mbar_arrive(mbar);
         }
         __syncwarp();
       } else {
         group_arrive(1 + grp);
       }
-      if (!__all_sync(FULL, mbar_wait(mbar, parity)) &&
-          !wait_agreed(mbar, parity, sh.wait_ns, &sh.gave_up[grp], kSplitGroup / 32, &sh.over)) {
-        // never seen, by any warp of the group: reported as a timeout
-        if (lane == 0) {
-          *(volatile int32_t *)&sh.lost[grp] = 1;
-          *(volatile int32_t *)&sh.lost_any = 1;
-          atomicExch(&sh.cdyn->err, 1);
-        }
-        __syncwarp();
-        if (i + 1 < steps) nearly();
-        return 0;
+      if (!__all_sync(FULL, mbar_wait(mbar, parity))) {
+        stop = kLost;
+        break;
       }
       stop = *(volatile int32_t *)&sh.stop[grp][parity];
       parity ^= 1u;
@@ -657,6 +611,27 @@ __device__ __forceinline__ unsigned long long task_split(const SlotDesc &sd, Spl
     }
     if (i + 1 < nst) stem_next<P, R, W, DB>(x, mult, l);
   }
+  if (stop == kLost) {
+    // This warp gives the product up.  The others of its group may have seen
+    // it in time: they get this warp's part in one more product (the named
+    // barrier's arrival; from the issuing warp the end of the product's phase)
+    // and leave by `stop` at the latest then.  No warp waits for this one but
+    // at the close, which all four come to whichever way.
+    if (lane == 0) {
+      *(volatile int32_t *)&sh.lost[grp] = 1;
+      *(volatile int32_t *)&sh.lost_any = 1;
+      atomicExch(&sh.cdyn->err, 1);
+      if ((warp & 3) == 0) {
+        *(volatile int32_t *)&sh.stop[grp][0] = 1;
+        *(volatile int32_t *)&sh.stop[grp][1] = 1;
+        mbar_arrive(mbar);
+        mbar_arrive(mbar);
+      }
+    }
+    __syncwarp();
+    if ((warp & 3) != 0) group_arrive(1 + grp);
+  }
+  group_sync(kCloseBar + grp);  // the close: after it, all four warps know of a loss (`lost`)
   return (unsigned long long)seen << (l > 0 ? 1 : 0);
 }
 
@@ -704,8 +679,6 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_sh.over = s_sh.lost_any = 0;
     for (int i = 0; i < kSplitGroups; ++i) s_sh.lost[i] = 0;
-    for (int i = 0; i <= kSplitGroups; ++i) s_sh.gave_up[i] = 0;
-    s_sh.wait_ns = kp.wait_limit_ns;
     s_sh.best_key = 0;
     s_sh.finished = 0;
     s_sh.states = states;
@@ -851,11 +824,16 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
     for (uint32_t n = 0;; ++n) {
       const int b = (int)(n & 1u);
       SplitTask &tk = s_sh.task[b];
-      if (!wait_agreed(smem_u32(&s_sh.full[n & 1u]), (n >> 1) & 1u, wait_ns, &s_sh.gave_up[kSplitGroups], kSplitWarps,
-                       &s_sh.over)) {  // no warp has anything more to wait for
-        atomicExch(&cdyn->err, 1);
-        break;
+      // the next task: the scheduler's waits are bounded, and it ends by an exit
+      // command or, where no buffer is free for one, by `over` (with nothing
+      // handed out after it: the warps leave at the same task)
+      bool have = false;
+      for (uint32_t r = 0; !have && r < (1u << 31); ++r) {
+        const bool over = *(volatile int32_t *)&s_sh.over;
+        have = __all_sync(0xffffffffu, mbar_test(smem_u32(&s_sh.full[n & 1u]), (n >> 1) & 1u));
+        if (__any_sync(0xffffffffu, over)) break;
       }
+      if (!have) break;
       if (tk.cmd == kCmdExit) break;
       if (tk.stage || tk.build) {
         if (tid == 0) tk.drop = *(volatile int32_t *)&s_sh.finished;
@@ -890,6 +868,8 @@ __global__ void __launch_bounds__(kSplitLaunch, 1)
       }
     }
   }
+  if (*(volatile int32_t *)&s_sh.lost_any)  // a product may still be under way: a millisecond for it before the tensor memory goes
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);
   tc_before_sync();
   __syncthreads();
   tc_after_sync();

@@ -16,11 +16,11 @@ def _same(a, b):
 @pytest.mark.gpu
 @pytest.mark.parametrize("p,n,k,budget", [(3, 80, 40, 0), (7, 52, 19, 3 * 10 ** 8), (5, 40, 20, 0)])
 def test_lost_product_ends_the_launch(p, n, k, budget):
-    """One warpgroup waits for an arrival that nobody makes: it gives up as a
-    whole after the wait limit, the other warps of its CTA are not left in a
-    barrier, and the same handle then gives the same result as before."""
+    """One warpgroup of each CTA waits for an arrival that nobody makes: it
+    gives up after about a second, the other warps of its CTA are not left in
+    a barrier, and the same handle then gives the same result as before."""
     code = inputs.single_code(400 + n, p, n, k)
-    o = B.fpcode_opts_default(budget=budget, mid_pass_exit=0, wait_limit_s=0.05)
+    o = B.fpcode_opts_default(budget=budget, mid_pass_exit=0)
     pr = B.fpcode_test_prepare_split(p, n, k, code.G, o)
     before = B.fpcode_min_distance_ex(pr, None, o)
     B.fpcode_test_lose_products(pr, True)
@@ -38,7 +38,7 @@ def test_lost_product_is_a_timeout(p, n, k, budget):
     """A task that was not compared in full is not counted off: the search
     reports a timeout, certifies nothing and claims no distance."""
     code = inputs.single_code(400 + n, p, n, k)
-    o = B.fpcode_opts_default(budget=budget, mid_pass_exit=0, wait_limit_s=0.05)
+    o = B.fpcode_opts_default(budget=budget, mid_pass_exit=0)
     pr = B.fpcode_test_prepare_split(p, n, k, code.G, o)
     whole = B.fpcode_min_distance_ex(pr, None, o)
     B.fpcode_test_lose_products(pr, True)
