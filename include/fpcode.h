@@ -138,7 +138,9 @@ typedef struct fpcode_result {
   int npasses;         /* passes entered (last pass index + 1) */
   int launch;          /* fpcode_min_distance_batch: index of the kernel
                           launch that searched this code (codes are grouped
-                          by kernel); t_kernel_ms is that launch's time */
+                          by kernel); t_kernel_ms is that launch's time,
+                          from its first CTA's start to its last one's end
+                          where several launches run side by side */
   int reserved1;
   uint64_t enumerated; /* codewords the GPU evaluated in the passes entered
                           (work taken ahead past the certifying pass is not

@@ -220,13 +220,14 @@ Layout make_layout(const std::vector<const fph::Prepared *> &codes) {
 // writes it there and zeroes the state for the next launch (else null: the
 // caller zeroes the state before and copies it back after each launch).
 void fill_static(const Layout &L, const std::vector<const fph::Prepared *> &codes, const DevCtx &c, char *h,
-                 char *d, int serve, char *outcome = nullptr) {
+                 char *d, int serve, char *outcome = nullptr, bool span = false) {
   CtlStatic cs{};
   cs.binom = c.binom;
   cs.aux = reinterpret_cast<fpk::SlotAux *>(d + L.off_aux);
   cs.slot_flags = reinterpret_cast<uint32_t *>(d + L.off_flags);
   cs.nslots = (int)codes.size();
   cs.serve = serve;
+  cs.span = span ? 1 : 0;
   if (outcome && codes.size() == 1 && !serve) {
     cs.outcome = outcome;
     cs.dyn_bytes = (uint32_t)L.dyn_bytes;
@@ -817,7 +818,7 @@ int fpcode_min_distance_batch(int num, const fpcode_desc *codes, void *stream, c
   };
   for (auto &g : ls) {
     char *d = c->ws + g.dev_off;
-    fill_static(g.L, g.codesv, *c, c->ws_pinned + g.pin_off, d, 0);
+    fill_static(g.L, g.codesv, *c, c->ws_pinned + g.pin_off, d, 0, nullptr, ls.size() > 1);
     if (!ok(cudaEventCreate(&g.e0)) || !ok(cudaEventCreate(&g.e1)) ||
         !ok(cudaMemcpyAsync(d, c->ws_pinned + g.pin_off, g.L.static_bytes, cudaMemcpyHostToDevice, st)) ||
         !ok(cudaMemsetAsync(d + g.L.off_states, 0, g.L.dyn_bytes + g.L.aux_bytes, st)))
@@ -853,6 +854,8 @@ int fpcode_min_distance_batch(int num, const fpcode_desc *codes, void *stream, c
       const SlotState *states = reinterpret_cast<const SlotState *>(c->ws_pinned + g.rb_off);
       CtlDyn dyn;
       std::memcpy(&dyn, c->ws_pinned + g.rb_off + g.L.dyn_bytes - sizeof(CtlDyn), sizeof(dyn));
+      // side by side, the event before a launch passes long before its first CTA gets an SM
+      if (dyn.end) ms = (float)((double)(dyn.end - ~dyn.begin) * 1e-6);
       for (size_t q = 0; q < g.idx.size(); ++q) {
         const int i = g.idx[q];
         uint8_t *w = witnesses ? witnesses + woff[i] : nullptr;

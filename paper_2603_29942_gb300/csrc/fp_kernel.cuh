@@ -46,6 +46,8 @@ struct CtlStatic {
   int32_t serve;          // serving: slots appear while the kernel runs
   uint32_t dyn_bytes;     // outcome: bytes of [SlotState][CtlDyn] copied out
   uint32_t clean_bytes;   // outcome: bytes of the dynamic state (states, aux, flags) zeroed for the next launch
+  int32_t span;           // 1: CtlDyn.begin and .end (launches that run side by side)
+  int32_t pad;
 };
 
 // A slot's flag word: (generation << 16) | kSlotFinished | kSlotExhausted.
@@ -75,6 +77,7 @@ struct CtlDyn {
   unsigned long long last_busy;  // serving: %globaltimer of a recent claim that found work (max over CTAs)
   uint32_t exited;  // one-code launches with an outcome copy: CTAs that have left
   uint32_t pad;
+  unsigned long long begin, end;  // CtlStatic.span: %globaltimer of the first CTA's start (inverted) and the last one's end
 };
 
 // Shared memory: binomial columns C(n, t), t < kBinomCols, then the staged
@@ -1770,6 +1773,10 @@ __global__ void __launch_bounds__(kThreads, FPK_MIN_BLOCKS) bz_kernel(const Slot
         slot_leave(cs, slot);
       }
     }
+  }
+  if (cs.span && tid == 0) {
+    atomicMax(&cdyn->begin, ~t_start);
+    atomicMax(&cdyn->end, globaltimer());
   }
   leave_launch(states, cs, cdyn);
 }

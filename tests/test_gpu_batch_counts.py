@@ -28,3 +28,18 @@ def test_enumerated_of_a_batch():
             pr = B.fpcode_prepare(c.p, c.n, c.k, c.G, B.fpcode_opts_default(budget=10 ** 7, pair_leaves=0))
             before = sum(ps[5] for ps in B.fpcode_prepared_passes(pr)[:int(r.field("npasses")[i]) - 1])
             assert r.field("enumerated")[i] >= before
+
+
+@pytest.mark.gpu
+def test_kernel_time_of_a_launch_is_its_own():
+    """Launches of one batch run side by side: a short one that waits for SMs
+    that a long one holds does not count the wait as its kernel time."""
+    long = inputs.single_code(21, 11, 60, 20)
+    short = [inputs.single_code(22 + i, 3, 24, 10) for i in range(4)]
+    o = B.fpcode_opts_default(budget=10 ** 10, mid_pass_exit=0)
+    for _ in range(3):
+        r = B.fpcode_min_distance_batch([long] + short, None, o)
+        launches = {x.launch for x in r[1:]}
+        assert len(launches) == 1 and r[0].launch not in launches
+        assert 0 < r[1].t_kernel_ms < 0.25 * r[0].t_kernel_ms
+        assert all(x.t_kernel_ms <= x.t_total_ms for x in r)
