@@ -1,5 +1,5 @@
 // fp_k_split.cu -- tensor-core enumeration kernels for one code with p = 3,
-// 5 or 7 (n - k up to 124 for p = 3, 45 for p = 5 and 7).
+// 5 or 7 (n - k up to 128 for p = 3, 42 for p = 5 and 7: split_k).
 #include "fp_split_kernel.cuh"
 #include "fp_kernels.h"
 

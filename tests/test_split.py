@@ -5,6 +5,7 @@ import math
 import numpy as np
 import pytest
 
+import oracle
 from paper_2603_29942_gb300 import _binding as B
 from paper_2603_29942_gb300 import inputs
 
@@ -130,3 +131,32 @@ def test_split_only_where_passes_are_large(p, n, k, split, lib):
     pr = B.fpcode_prepare(p, n, k, code.G, B.fpcode_opts_default())
     last = max(i for i, ps in enumerate(B.fpcode_prepared_schedule(pr)) if ps["g"] <= 3)
     assert (B.fpcode_test_split_pass(pr, last, cap=1 << 16) is not None) is split
+
+
+# the widest rows of p = 3 (n - k = 128: 124 positions compared), and of p = 5 and 7 (n - k = 42)
+ORACLE_CODES = [(3, 140, 12), (3, 139, 11), (3, 138, 12), (3, 137, 13), (3, 60, 20), (5, 53, 11), (5, 30, 12), (7, 53, 11),
+                (7, 33, 9)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("p,n,k", ORACLE_CODES)
+def test_split_search_equals_oracle(p, n, k):
+    """Interval, schedule and counts as the oracle's, every pass in full, and
+    a witness of the best weight."""
+    code = inputs.single_code(1700 + n, p, n, k)
+    o = B.fpcode_opts_default(budget=3 * 10 ** 6, mid_pass_exit=0)
+    pr = B.fpcode_test_prepare_split(p, n, k, code.G, o)
+    a = B.fpcode_min_distance_ex(pr, None, o)
+    b = oracle.bz(code, threads=4, budget=3 * 10 ** 6)
+    assert {oracle.OK: B.OK, oracle.EBUDGET: B.EBUDGET}[b.status] == a.status
+    assert (a.L, a.U) == (b.L, b.U) and list(a.counts) == list(b.counts)
+    assert a.enumerated == sum(a.counts)
+    assert np.count_nonzero(np.array(a.witness)) == a.U
+
+
+@pytest.mark.parametrize("p,most", [(3, 128), (5, 42), (7, 42)])
+def test_widest_split_rows(p, most, lib):
+    """Redundant symbols up to which the class values fit a row."""
+    assert _prep(inputs.single_code(5, p, 20 + most, 20)) is not None
+    if most < 128:
+        assert _prep(inputs.single_code(5, p, 21 + most, 20)) is None
