@@ -253,7 +253,7 @@ FP_HD uint32_t lookup(const uint32_t *a) {
 template <int P, int R>
 struct ClassLog {
   static_assert(P == (1 << R) - 1 && (P == 31 || P == 127), "3 is a primitive root");
-  static constexpr uint64_t table(int bit) {
+  FP_HD static constexpr uint64_t table(int bit) {
     uint64_t t = 0;
     int v = 1;
     for (int e = 0; e < (P - 1) / 2; ++e, v = v * 3 % P)

@@ -672,16 +672,16 @@ __device__ __noinline__ void build_labels(uint32_t *tab, int k, int p) {
 #pragma unroll
       for (int z = W * R; z < RWP; ++z) o[z] = 0u;
     }
-    return;
-  }
-  for (int i = threadIdx.x; i < k * np; i += kThreads) {
-    const int t = i / np, q = i - t * np;
-    const uint32_t *e = tab + (t * (p - 1) + q) * RWP;
-    uint32_t *o = lab + i * LS;
+  } else {
+    for (int i = threadIdx.x; i < k * np; i += kThreads) {
+      const int t = i / np, q = i - t * np;
+      const uint32_t *e = tab + (t * (p - 1) + q) * RWP;
+      uint32_t *o = lab + i * LS;
 #pragma unroll
-    for (int w = 0; w < W; ++w) fpbs::class_label<P, R>(e + w * R, o + w * (R - 1), p);
+      for (int w = 0; w < W; ++w) fpbs::class_label<P, R>(e + w * R, o + w * (R - 1), p);
 #pragma unroll
-    for (int z = W * (R - 1); z < LS; ++z) o[z] = 0u;
+      for (int z = W * (R - 1); z < LS; ++z) o[z] = 0u;
+    }
   }
 }
 

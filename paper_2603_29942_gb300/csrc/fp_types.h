@@ -94,11 +94,19 @@ FPK_HD int label_words(int p, int r, int W) { return p == 5 ? W * (r - 1) : (W *
 // Labels are kept while a lane's sum and its label leave room in 64
 // registers (beyond: spills), and while they fit behind the multiples.
 FPK_HD constexpr bool label_shape(int r, int W) { return W * (2 * r - 1) <= 36; }
-// p = 31 and 127 with at most 64 redundant positions (beyond: spills) keep
-// one entry a row instead: the logarithm of its class (fp_kernel.cuh).
+// p = 31 and 127 with at most 64 redundant positions keep one entry a row
+// instead: the logarithm of its class (fp_kernel.cuh).  At two words p = 127
+// spills 692 bytes a thread (p = 31: 296) and is faster all the same (F_127
+// [70,6] 488 us, 530 with labels).  At three and four words p = 31 would spill
+// 696 and 812 (216 and 380 with labels), and p = 127 has no labels to replace.
 FPK_HD constexpr bool log_labels(int p, int W) { return (p == 31 || p == 127) && W <= 2; }
 // Words of an information set's labels; 0: none (p = 3 and 7 have row
-// signatures, and sets that would not fit take the two subtractions).
+// signatures, and sets that would not fit take the two subtractions).  They
+// are taken also where their shared memory leaves fewer CTAs an SM (p = 11,
+// k = 64, three words: three for four; p = 17, k = 64, two words: two for
+// three): kernel, two subtractions against labels, F_11 [144,64] 165 and 127
+// us, F_11 [130,64] 170 and 124, F_17 [114,64] 210 and 163, F_13 [150,60] 175
+// and 134; none of 30 shapes over p = 5 .. 251 was slower.
 FPK_HD int set_label_words(int p, int r, int W, int k) {
   if (p == 3 || p == 7 || !label_shape(r, W)) return 0;
   const int rwp = (r * W + 3) & ~3;
