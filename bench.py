@@ -80,12 +80,12 @@ FLUSH_BYTES = 256 << 20
 # (the hash skips comments and blank lines).
 KERNEL_SOURCES = ["fp_kernel.cuh", "fp_enum.cuh", "fp_bitslice.cuh", "fp_types.h", "fp_split.cuh",
                   "fp_split_kernel.cuh"]
-_SHA_PROFILED = "8780d0da516689b5a57dcd3df7282efb232c48e9f0263d9e0ea74675ba62254a"
-PROFILED_TRAFFIC: dict = {  # profiles/bz_kernel_*.md (the command of each capture is there)
-    "f3_n80_k40": {"bytes": 5725952 + 0, "sources_sha256": _SHA_PROFILED},
-    "probe_f3_n80_k40_g8": {"bytes": 5715712 + 0, "sources_sha256": _SHA_PROFILED},
-    "f7_n40_k20": {"bytes": 9477376 + 256, "sources_sha256": _SHA_PROFILED},
-    "probe_f7_n40_k20_g7": {"bytes": 7579136 + 29952, "sources_sha256": _SHA_PROFILED},
+_SHA_PROFILED = "caeaea147c1a389f38905fc5756c196d1a4bfb8c0fc4a8d1a32766892965e886"
+PROFILED_TRAFFIC: dict = {  # profiles/*_kernel_*.md (the command of each capture is there)
+    "f3_n80_k40": {"bytes": 335616 + 2304, "sources_sha256": _SHA_PROFILED},
+    "probe_f3_n80_k40_g8": {"bytes": 5716224 + 0, "sources_sha256": _SHA_PROFILED},
+    "f7_n40_k20": {"bytes": 9479424 + 0, "sources_sha256": _SHA_PROFILED},
+    "probe_f7_n40_k20_g7": {"bytes": 7579904 + 35072, "sources_sha256": _SHA_PROFILED},
 }
 
 
