@@ -35,10 +35,10 @@
 // the steps).  Three warpgroups of N = 128, or of two N = 64 accumulators,
 // and two half-size table buffers were slower.
 //
-// Against the popcount kernels (whole search): F_3 [80,40] 174 -> 119 us,
-// F_7 [50,25] 845 -> 302, F_7 [52,19] 17389 -> 1965, F_3 [74,50] 1254 ->
-// 372, F_5 [51,24] 431 -> 126.  ncu, F_7 [50,25]: tensor pipe 23 %, ALU 41 %,
-// issue slots 37 %: bound by latency within a step, not by a pipe.
+// Against the popcount kernels (whole search): F_3 [80,40] 174 -> 120 us,
+// F_7 [50,25] 845 -> 301, F_7 [52,19] 17389 -> 1940, F_3 [74,50] 1254 ->
+// 375, F_5 [51,24] 431 -> 126.  ncu, F_7 [50,25]: tensor pipe 24 %, ALU 41 %,
+// issue slots 38 %: bound by latency within a step, not by a pipe.
 #pragma once
 #include "fp_kernel.cuh"
 #include "fp_split.cuh"
