@@ -740,7 +740,10 @@ void plan_tasks(Prepared *P, int ctas, int fixed_pl, int min_steps, bool spread_
     // default of one code: where up to four units a lane fill the grid, all of
     // it (kernel times, eight steps against the rule: F_3 [43,23] 38.7 and
     // 28.5 us, F_31 [32,7] 43.0 and 35.7); F_7 [40,20] at six a lane instead
-    // of eight on two thirds of the grid took 46.7 us, not 45.0
+    // of eight on two thirds of the grid took 46.7 us, not 45.0.  (The other way
+    // round where a search ends while such a pass is taken ahead and the tasks
+    // run on to their next look at the flag: F_3 [54,43], mid_pass_exit 0, 47.4
+    // and 50.5.)
     const uint64_t fill = (N + lanes * C - 1) / (lanes * C);
     if (min_steps <= 0 && fill <= 4) umin = std::min(umin, std::max<uint64_t>(1, fill));
     if (spread_tiny && N <= lanes * C) {  // under one unit per lane of the grid: spread it wide
